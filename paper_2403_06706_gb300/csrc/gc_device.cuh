@@ -13,6 +13,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "gc_f32x2.cuh"
 #include "unit_circle_table.h"
 
 namespace gcp {
@@ -216,49 +217,6 @@ __device__ __forceinline__ void load_node_pairs(const float *p, unsigned long lo
     asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
         : "=l"(q[0]), "=l"(q[1]), "=l"(q[2]), "=l"(q[3])
         : "l"(p));
-}
-
-// Two FP32 channels in one 64-bit register and the packed f32x2 arithmetic of sm_100+ (two
-// independent IEEE operations per instruction, the same results as two scalar ones).
-__device__ __forceinline__ unsigned long long p2_sub(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long p2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long p2_bcast(float x)
-{
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long p2_pack(float lo, float hi)
-{
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long p2_mul(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ void p2_split(unsigned long long v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
 
 // The trilinear interpolant of one node array at a located point (cell offsets o0 / o1 of

@@ -7,8 +7,8 @@
 // (r / 1 AU) / E_scale, Phi / (E_scale 1 AU). The training minimises the mean squared error
 // over samples and channels (Kingma & Ba 2015 for Adam) with the same arithmetic as the
 // fused evaluation: W2..W5 and the activations h_1..h_4 in BF16, FP32 accumulation, FP32
-// first layer and biases. Products with W2..W4 (forward, dW = dZ^T H, dH = dZ W) run on the
-// tensor-core GEMM; the first and last layers and the elementwise steps run here.
+// first layer and biases. The forward and backward passes are in gc_train.cu; the targets,
+// Adam and the parameters' BF16 copies are here.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -58,14 +58,15 @@ __global__ void k_to_bf16(const float *__restrict__ P, __nv_bfloat16 *Wh, __nv_b
         put_bf16(i, P[i], Wh, W5p);
 }
 
-// Adam (Kingma & Ba 2015) with bias corrections bc1 = 1 - beta1^t, bc2 = 1 - beta2^t
-__global__ void k_adam(float *__restrict__ P, const float *__restrict__ G, float *__restrict__ M,
+// Adam (Kingma & Ba 2015) with bias corrections bc1 = 1 - beta1^t, bc2 = 1 - beta2^t; clears G
+__global__ void k_adam(float *__restrict__ P, float *__restrict__ G, float *__restrict__ M,
                        float *__restrict__ V, float lr, float b1, float b2, float eps, float bc1, float bc2,
                        __nv_bfloat16 *Wh, __nv_bfloat16 *W5p)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < kSirenNParams;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float g = G[i];
+        G[i] = 0.f; // the next batch adds to it
         const float m = b1 * M[i] + (1.0f - b1) * g;
         const float v = b2 * V[i] + (1.0f - b2) * g * g;
         M[i] = m;
@@ -124,187 +125,6 @@ __global__ void k_targets(const T *__restrict__ nodes, int n_r, int n_th, int n_
     }
 }
 
-// first layer: z1 = w0 (W1 x + b1), h1 = sin z1 (rows x 256)
-__global__ void k_layer1(const float *__restrict__ P, const float *__restrict__ x, int64_t n, float w0,
-                         float *__restrict__ Z, __nv_bfloat16 *__restrict__ H)
-{
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n * 256;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = q >> 8;
-        const int f = (int)(q & 255);
-        const float *w = P + siren_oW(1) + 3 * f;
-        const float z = w0 * fmaf(w[0], x[3 * row], fmaf(w[1], x[3 * row + 1], fmaf(w[2], x[3 * row + 2],
-                                                                                      P[siren_oB(1) + f])));
-        Z[q] = z;
-        H[q] = __float2bfloat16_rn(sinf(z));
-    }
-}
-
-// hidden layer L: z = (W_L h)_GEMM + b_L in place, h_L = sin z
-__global__ void k_act(const float *__restrict__ P, int L, int64_t n, float *__restrict__ Z,
-                      __nv_bfloat16 *__restrict__ H)
-{
-    const float *b = P + siren_oB(L);
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n * 256;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const float z = Z[q] + b[q & 255];
-        Z[q] = z;
-        H[q] = __float2bfloat16_rn(sinf(z));
-    }
-}
-
-// Output layer forward and its backward: y = W5 h4 + b5, r = y - t, loss += sum r^2,
-// dy = gscale r, dW5 += dy h4^T, db5 += dy, dz4 = (W5^T dy) cos z4, db4 += dz4. One warp
-// per sample (lane: features 8 lane .. 8 lane + 7); block sums go to the gradient by atomics.
-__global__ void __launch_bounds__(256) k_out(const float *__restrict__ P, const __nv_bfloat16 *__restrict__ W5p,
-                                             const __nv_bfloat16 *__restrict__ H4, const float *__restrict__ Z4,
-                                             const float *__restrict__ T, int64_t n, float gscale,
-                                             __nv_bfloat16 *__restrict__ dZ4, float *__restrict__ G,
-                                             double *__restrict__ loss)
-{
-    __shared__ float sW[8][256];
-    __shared__ float sAcc[2048 + 256 + 8];
-    __shared__ double sLoss[8];
-    for (int i = threadIdx.x; i < 2048; i += 256)
-        sW[i >> 8][i & 255] = __bfloat162float(W5p[i]);
-    for (int i = threadIdx.x; i < 2048 + 264; i += 256)
-        sAcc[i] = 0.f;
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, f0 = lane * 8;
-    float b5[8];
-#pragma unroll
-    for (int o = 0; o < 8; ++o)
-        b5[o] = P[siren_oB(5) + o];
-    float aW[8][8], aB4[8], aB5[8];
-#pragma unroll
-    for (int o = 0; o < 8; ++o) {
-        aB4[o] = 0.f;
-        aB5[o] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            aW[o][i] = 0.f;
-    }
-    double ls = 0.0;
-    for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < n; row += (int64_t)gridDim.x * 8) {
-        const uint4 hv = *reinterpret_cast<const uint4 *>(H4 + row * 256 + f0);
-        const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&hv);
-        float h[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 t2 = __bfloat1622float2(h2[i]);
-            h[2 * i] = t2.x;
-            h[2 * i + 1] = t2.y;
-        }
-        float part[8];
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-            float a = 0.f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                a = fmaf(sW[o][f0 + i], h[i], a);
-            part[o] = a;
-        }
-#pragma unroll
-        for (int o = 0; o < 8; ++o)
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1)
-                part[o] += __shfl_xor_sync(0xffffffffu, part[o], off);
-        float dy[8];
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-            const float r = part[o] + b5[o] - T[row * 8 + o];
-            if (lane == 0) ls += (double)r * (double)r;
-            dy[o] = gscale * r;
-            aB5[o] += dy[o];
-        }
-        const float4 za = *reinterpret_cast<const float4 *>(Z4 + row * 256 + f0);
-        const float4 zb = *reinterpret_cast<const float4 *>(Z4 + row * 256 + f0 + 4);
-        const float zz[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
-        float dz[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float dh = 0.f;
-#pragma unroll
-            for (int o = 0; o < 8; ++o) {
-                dh = fmaf(dy[o], sW[o][f0 + i], dh);
-                aW[o][i] = fmaf(dy[o], h[i], aW[o][i]);
-            }
-            dz[i] = dh * cosf(zz[i]);
-            aB4[i] += dz[i];
-        }
-        uint4 pk;
-        __nv_bfloat162 p0 = __floats2bfloat162_rn(dz[0], dz[1]), p1 = __floats2bfloat162_rn(dz[2], dz[3]),
-                       p2 = __floats2bfloat162_rn(dz[4], dz[5]), p3 = __floats2bfloat162_rn(dz[6], dz[7]);
-        pk.x = *reinterpret_cast<uint32_t *>(&p0);
-        pk.y = *reinterpret_cast<uint32_t *>(&p1);
-        pk.z = *reinterpret_cast<uint32_t *>(&p2);
-        pk.w = *reinterpret_cast<uint32_t *>(&p3);
-        *reinterpret_cast<uint4 *>(dZ4 + row * 256 + f0) = pk;
-    }
-    for (int w = 0; w < 8; ++w) {
-        if (warp == w) {
-#pragma unroll
-            for (int o = 0; o < 8; ++o)
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    sAcc[o * 256 + f0 + i] += aW[o][i];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                sAcc[2048 + f0 + i] += aB4[i];
-            if (lane == 0)
-#pragma unroll
-                for (int o = 0; o < 8; ++o)
-                    sAcc[2304 + o] += aB5[o];
-        }
-        __syncthreads();
-    }
-    if (lane == 0) sLoss[warp] = ls;
-    __syncthreads();
-    for (int i = threadIdx.x; i < 2048; i += 256)
-        atomicAdd(G + siren_oW(5) + i, sAcc[i]);
-    atomicAdd(G + siren_oB(4) + threadIdx.x, sAcc[2048 + threadIdx.x]);
-    if (threadIdx.x < 8) atomicAdd(G + siren_oB(5) + threadIdx.x, sAcc[2304 + threadIdx.x]);
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w)
-            t += sLoss[w];
-        atomicAdd(loss, t);
-    }
-}
-
-// dz_L = dh_L cos z_L (BF16 for the next products) and db_L += sum over rows; for the
-// first layer dz_1 = w0 dh_1 cos z_1, dW1 += dz_1 x^T, db1 += dz_1 instead. Thread = feature,
-// block = a slab of rows.
-__global__ void __launch_bounds__(256) k_bwd_act(const float *__restrict__ dH, const float *__restrict__ Z,
-                                                 int64_t n, int rows_per_block, int L, float w0,
-                                                 const float *__restrict__ x, __nv_bfloat16 *__restrict__ dZ,
-                                                 float *__restrict__ G)
-{
-    const int f = threadIdx.x;
-    const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-    const int64_t r1 = r0 + rows_per_block < n ? r0 + rows_per_block : n;
-    float acc = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f;
-    for (int64_t row = r0; row < r1; ++row) {
-        const int64_t q = row * 256 + f;
-        float d = dH[q] * cosf(Z[q]);
-        if (L == 1) {
-            d *= w0;
-            a0 = fmaf(d, x[3 * row], a0);
-            a1 = fmaf(d, x[3 * row + 1], a1);
-            a2 = fmaf(d, x[3 * row + 2], a2);
-        } else {
-            dZ[q] = __float2bfloat16_rn(d);
-        }
-        acc += d;
-    }
-    atomicAdd(G + siren_oB(L) + f, acc);
-    if (L == 1) {
-        atomicAdd(G + siren_oW(1) + 3 * f, a0);
-        atomicAdd(G + siren_oW(1) + 3 * f + 1, a1);
-        atomicAdd(G + siren_oW(1) + 3 * f + 2, a2);
-    }
-}
-
 template <typename P>
 cudaError_t dev_alloc(P **p, size_t bytes)
 {
@@ -314,19 +134,11 @@ cudaError_t dev_alloc(P **p, size_t bytes)
 cudaError_t ensure_work(Neural &nn, int64_t rows)
 {
     if (rows <= nn.wcap) return cudaSuccess;
-    cudaFree(nn.Z);
-    cudaFree(nn.H);
-    cudaFree(nn.dZ);
-    cudaFree(nn.dH);
-    nn.Z = nullptr;
-    nn.H = nullptr;
-    nn.dZ = nullptr;
-    nn.dH = nullptr;
+    cudaFree(nn.act);
+    nn.act = nullptr;
     nn.wcap = 0;
-    cudaError_t e = dev_alloc(&nn.Z, (size_t)4 * rows * 256 * sizeof(float));
-    if (e == cudaSuccess) e = dev_alloc(&nn.H, (size_t)4 * rows * 256 * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = dev_alloc(&nn.dZ, (size_t)rows * 256 * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = dev_alloc(&nn.dH, (size_t)rows * 256 * sizeof(float));
+    cudaError_t e = dev_alloc(&nn.act, (size_t)6 * 256 * rows * sizeof(__nv_bfloat16));
+    if (e == cudaSuccess) e = gcs::train_act_map(&nn.map_act, nn.act, rows);
     if (e == cudaSuccess) nn.wcap = rows;
     return e;
 }
@@ -334,44 +146,15 @@ cudaError_t ensure_work(Neural &nn, int64_t rows)
 // forward and backward of one batch; adds sum r^2 to nn.d_loss and the gradient to grad
 cudaError_t fwd_bwd(Neural &nn, const float *x, const float *t, int64_t n, float *grad, cudaStream_t s)
 {
-    cudaError_t e = ensure_work(nn, n);
-    if (e != cudaSuccess) return e;
-    const size_t slab = (size_t)nn.wcap * 256;
-    float *Z[4];
-    __nv_bfloat16 *H[4];
-    for (int k = 0; k < 4; ++k) {
-        Z[k] = nn.Z + k * slab;
-        H[k] = nn.H + k * slab;
-    }
-    const float w0 = (float)nn.omega0;
-    const int eb = blocks_for(n * 256, 256);
-    k_layer1<<<eb, 256, 0, s>>>(nn.P, x, n, w0, Z[0], H[0]);
-    for (int L = 2; L <= 4; ++L) {
-        e = gcs::gemm_bf16(H[L - 2], 0, nn.Wh + (size_t)(L - 2) * 65536, 0, Z[L - 1], (int)n, 256, 256, 1, 0, s);
-        if (e != cudaSuccess) return e;
-        k_act<<<eb, 256, 0, s>>>(nn.P, L, n, Z[L - 1], H[L - 1]);
-    }
-    k_out<<<blocks_for(n, 8, 152 * 4), 256, 0, s>>>(nn.P, nn.W5p, H[3], Z[3], t, n, (float)(2.0 / (double)(n * 8)),
-                                                    nn.dZ, grad, nn.d_loss);
-    // K = n split so that about two waves of CTAs share each dW product
-    const int splits = (int)std::max<int64_t>(1, std::min<int64_t>(n / 64, 152));
-    const int rows_per_block = 32;
-    const int bb = (int)((n + rows_per_block - 1) / rows_per_block);
-    for (int L = 4; L >= 2; --L) {
-        e = gcs::gemm_bf16(nn.dZ, 1, H[L - 2], 1, grad + siren_oW(L), 256, 256, (int)n, splits, 1, s);
-        if (e != cudaSuccess) return e;
-        e = gcs::gemm_bf16(nn.dZ, 0, nn.Wh + (size_t)(L - 2) * 65536, 1, nn.dH, (int)n, 256, 256, 1, 0, s);
-        if (e != cudaSuccess) return e;
-        k_bwd_act<<<bb, 256, 0, s>>>(nn.dH, Z[L - 2], n, rows_per_block, L - 1, w0, x, nn.dZ, grad);
-    }
-    return cudaGetLastError();
+    const cudaError_t e = ensure_work(nn, n);
+    return e != cudaSuccess ? e : gcs::train_fwd_bwd(nn.net, nn.map_act, x, t, n, grad, nn.d_loss, s);
 }
 
 } // namespace
 
 cudaError_t neural_free(Neural &nn)
 {
-    void *ptrs[] = {nn.P, nn.G, nn.Mo, nn.Vo, nn.Wh, nn.W5p, nn.Z, nn.H, nn.dZ, nn.dH, nn.d_loss, nn.d_err, nn.Xs, nn.Ts};
+    void *ptrs[] = {nn.P, nn.G, nn.Mo, nn.Vo, nn.Wh, nn.W5p, nn.act, nn.d_loss, nn.d_err, nn.Xs, nn.Ts};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     nn = Neural{};
@@ -528,11 +311,11 @@ cudaError_t neural_fit(Neural &nn, const GridRef &g, const float *samples, bool 
     if (e == cudaSuccess) e = neural_targets(nn, g, nn.Xs, n_samples, nn.Ts, s);
     if (e != cudaSuccess) return e;
     const int64_t nb = n_samples / batch;
+    e = cudaMemsetAsync(nn.G, 0, (size_t)kSirenNParams * sizeof(float), s);
     for (int ep = 0; ep < n_epochs; ++ep) {
-        e = cudaMemsetAsync(nn.d_loss, 0, sizeof(double), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(nn.d_loss, 0, sizeof(double), s);
         for (int64_t b = 0; b < nb && e == cudaSuccess; ++b) {
-            e = cudaMemsetAsync(nn.G, 0, (size_t)kSirenNParams * sizeof(float), s);
-            if (e == cudaSuccess) e = fwd_bwd(nn, nn.Xs + b * batch * 3, nn.Ts + b * batch * 8, batch, nn.G, s);
+            e = fwd_bwd(nn, nn.Xs + b * batch * 3, nn.Ts + b * batch * 8, batch, nn.G, s);
             if (e == cudaSuccess) e = neural_adam(nn, lr, beta1, beta2, eps, s);
         }
         if (e != cudaSuccess) return e;

@@ -31,14 +31,12 @@ struct Neural {
     double omega0 = 30.0, r_max = 0.0, B_scale = 1.0, E_scale = 1.0;
     int64_t adam_t = 0;
 
-    // per-batch work buffers of the training (rows = samples)
+    // work buffer of the training: h1..h3 and dz2..dz4 of a batch, [6][256][wcap] BF16
     int64_t wcap = 0;
-    float *Z = nullptr;          // 4 x wcap x 256 pre-activations z_1..z_4
-    __nv_bfloat16 *H = nullptr;  // 4 x wcap x 256 activations h_1..h_4
-    __nv_bfloat16 *dZ = nullptr; // wcap x 256
-    float *dH = nullptr;         // wcap x 256
+    __nv_bfloat16 *act = nullptr;
+    CUtensorMap map_act{};
     double *d_loss = nullptr;    // [1]
-    int *d_err = nullptr;        // error word of the fused evaluation
+    int *d_err = nullptr;        // error word of the fused evaluation and training
 
     // fit: samples and targets
     float *Xs = nullptr, *Ts = nullptr;

@@ -63,6 +63,12 @@ struct SirenIn {
 cudaError_t siren_maps(SirenNet &net);
 // evaluate the network (and its Jacobian) at the input points (device)
 cudaError_t siren_eval(const SirenNet &net, const SirenIn &in, const SirenOut &out, cudaStream_t s);
+// Training (gc_train.cu): adds the gradient of the mean squared error of n samples (n a
+// multiple of 64) to G and the sum of squared residuals to loss. act: tensor map, made by
+// train_act_map, of a BF16 work buffer of 6 x 256 rows of `cap` >= n samples (h1..h3, dz2..dz4).
+cudaError_t train_act_map(CUtensorMap *m, const void *act, int64_t cap);
+cudaError_t train_fwd_bwd(const SirenNet &net, const CUtensorMap &act, const float *x, const float *t, int64_t n,
+                          float *G, double *loss, cudaStream_t s);
 // CTAs of the fused evaluation per launch (one per SM)
 int siren_eval_grid(int64_t n);
 } // namespace gcs

@@ -72,12 +72,6 @@ struct EvalParams {
     int *err;        // error word (device), set when a wait runs out
 };
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
-{
-    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t *>(&v);
-}
-
 // 8 consecutive rows (mn0 .. mn0 + 7, mn0 % 8 == 0) of one feature into the MN-major
 // activation buffer; hrow points at the feature's 128-byte row of its K-group's first atom
 __device__ __forceinline__ void store_rows8(uint8_t *hrow, uint32_t rsw, uint32_t mn0, const float (&o)[8])
@@ -89,22 +83,6 @@ __device__ __forceinline__ void store_rows8(uint8_t *hrow, uint32_t rsw, uint32_
     pk.w = pack_bf16(o[6], o[7]);
     const uint32_t ch = ((mn0 & 63u) >> 3) ^ rsw;
     *reinterpret_cast<uint4 *>(hrow + (mn0 >> 6) * 1024u + ch * 16u) = pk;
-}
-
-// bounded wait that also gives up when another role of the CTA has aborted
-__device__ __forceinline__ bool wait_abort(uint64_t *bar, uint32_t parity, volatile int *abort, int *err, int code)
-{
-    if (mbar_try(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    for (;;) {
-        for (int i = 0; i < 32; ++i)
-            if (mbar_try(bar, parity)) return true;
-        if (*abort) return false;
-        if (global_ns() - t0 > kWaitNs) break;
-    }
-    *abort = 1;
-    atomicExch(err, code);
-    return false;
 }
 
 // Output rows of one tile from the output accumulator v (16 columns of this thread's row

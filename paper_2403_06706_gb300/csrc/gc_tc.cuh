@@ -10,6 +10,7 @@
 
 #include <cstdint>
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 namespace tc {
@@ -79,6 +80,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity)
     }
 }
 
+// Bounded wait that also gives up when another role of the CTA has aborted; one that runs out
+// sets the CTA's abort flag and the kernel's error word.
+__device__ __forceinline__ bool wait_abort(uint64_t *bar, uint32_t parity, volatile int *abort, int *err, int code)
+{
+    if (mbar_try(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    for (;;) {
+        for (int i = 0; i < 32; ++i)
+            if (mbar_try(bar, parity)) return true;
+        if (*abort) return false;
+        if (global_ns() - t0 > kWaitNs) break;
+    }
+    *abort = 1;
+    atomicExch(err, code);
+    return false;
+}
+
 // ---------------------------------------------------------------------------- TMA
 // 2-D tile load: coordinates (inner element index, outer row index); inner must be a
 // multiple of 8 bf16 (16 bytes).
@@ -90,6 +108,22 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
                  "l"((uint64_t)map), "r"(inner), "r"(outer), "r"(smem_u32(bar))
                  : "memory");
 }
+
+// 2-D tile store shared -> global (bulk group of the issuing thread). Writers of the tile have
+// made their stores visible with fence_proxy_async_smem().
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int32_t inner, int32_t outer, const void *src)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     (uint64_t)map),
+                 "r"(inner), "r"(outer), "r"(smem_u32(src))
+                 : "memory");
+}
+
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+
+// every committed bulk store of this thread has read its source / is complete
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // contiguous bulk copy global -> shared (16-byte aligned, size a multiple of 16)
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
@@ -177,6 +211,25 @@ __device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t smem_addr, uint32_t l
     return d;
 }
 
+// The two words of those descriptors apart, for issue loops: the high word (stride and
+// layout) is a constant of the operand, the low one moves by bytes / 16 within it.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr, uint32_t lbo)
+{
+    return ((smem_addr & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16);
+}
+
+__host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14) | (2u << 29); }
+
+__device__ __forceinline__ uint64_t desc_of(uint32_t hi, uint32_t lo) { return (uint64_t)hi << 32 | lo; }
+
+// one lane of a converged warp (the same one every time)
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 // Instruction descriptor: BF16 x BF16 -> FP32, M x N; a_mn / b_mn select MN-major operands
 // (0 = K-major).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn = 0, int b_mn = 0)
@@ -218,6 +271,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 #pragma unroll
     for (int i = 0; i < 16; ++i)
         v[i] = __uint_as_float(r[i]);
+}
+
+// Store 16 consecutive 32-bit columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+                 "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]),
+                 "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+                 : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
+{
+    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t *>(&v);
 }
 
 // byte offset of element (row, k) (k < 64, bf16) inside an 8-row-atom K-major SW128 tile
