@@ -207,114 +207,123 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == kTmaWarp) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            uint32_t g = 0;
+            uint32_t st = 0, par = 1, filled = 0;
             bool ok = true;
             mbar_expect_tx(w5full, kW5Bytes);
             for (int kb = 0; kb < 4; ++kb)
                 tma_load_2d(sW5 + kb * 2048, &mw5, kb * 64, 0, w5full);
             for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+#pragma unroll 1
                 for (int c = 0; c < kChunksPerTile; ++c) {
-                    const uint32_t s = g % kStagesW;
-                    if (!wait_abort(&empty[s], ((g / kStagesW) & 1u) ^ 1u, abort, p.err, 11)) {
+                    if (!wait_abort(&empty[st], par, abort, p.err, 11)) {
                         ok = false;
                         break;
                     }
-                    uint8_t *dst = sW + s * kChunkBytes;
                     // chunk (layer c / 8, output half and input block in the MMA order)
                     const int q = c & 7, h = (q >> 1) & 1, kb = (q & 1) | ((q >> 2) << 1);
-                    mbar_expect_tx(&full[s], kChunkBytes);
-                    tma_load_2d(dst, &mwh, kb * 64, (c >> 3) * 256 + h * 128, &full[s]);
-                    ++g;
+                    mbar_expect_tx(&full[st], kChunkBytes);
+                    tma_load_2d(sW + st * kChunkBytes, &mwh, kb * 64, (c >> 3) * 256 + h * 128, &full[st]);
+                    filled |= 1u << st;
+                    if (++st == kStagesW) {
+                        st = 0;
+                        par ^= 1u;
+                    }
                 }
             }
-            // the copies still in flight land before the CTA's shared memory is released
-            for (uint32_t j = g > (uint32_t)kStagesW ? g - kStagesW : 0u; j < g; ++j)
-                mbar_wait(&full[j % kStagesW], (j / kStagesW) & 1u);
+            // the copies still in flight land before the CTA's shared memory is released: the
+            // last copy of a stage behind st is of the running phase, of one from st on of the
+            // phase before
+            for (int j = 0; j < kStagesW; ++j)
+                if (filled >> j & 1)
+                    mbar_wait(&full[j], (uint32_t)j < st ? par ^ 1u : par);
             mbar_wait(w5full, 0);
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t id_hid = idesc_bf16_f32(128, 256, 0, 1);
-            const uint32_t id_out = idesc_bf16_f32(128, 16, 1, 0);
-            const uint32_t hb = smem_u32(sH);
-            uint32_t g = 0, nh0 = 0, nh1 = 0, nd = 0;
-            bool ok = true;
-            for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-                for (int L = 0; L < 3 && ok; ++L) {
-                    // order: half 0 over inputs 0-127, half 1 over inputs 0-127 (as soon as the
-                    // previous half-1 epilogue has read its accumulator), half 0 over 128-255
-                    // (once that epilogue has written them), half 1 over 128-255
+        // The whole warp runs the loop and one elected lane issues; descriptors are a constant
+        // high word and a running low word. With descriptors built from addresses for every MMA
+        // and the stage found by a division, beside four compute warps on the same scheduler an
+        // MMA took 170 cycles to issue against the 128 the tensor cores need for it.
+        constexpr uint32_t id_hid = idesc_bf16_f32(128, 256, 0, 1);
+        constexpr uint32_t id_out = idesc_bf16_f32(128, 16, 1, 0);
+        const bool leader = elect_one();
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t h_lo = desc_lo(smem_u32(sH), 1024), w_lo = desc_lo(smem_u32(sW), 16);
+        uint32_t st = 0, par = 0, nh = 0, nd = 0; // ring stage and its phase, operands, drains
+        bool ok = true;
+        auto wait = [&](uint64_t *bar, uint32_t phase, int code) {
+            const bool r = __all_sync(0xffffffffu, wait_abort(bar, phase & 1u, abort, p.err, code)) != 0;
+            tc_fence_after();
+            return r;
+        };
+        // W5, loaded once per launch
+        if (blockIdx.x < n_tiles) ok = wait(w5full, 0, 17);
+        for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
 #pragma unroll 1
-                    for (int q = 0; q < 8; ++q) {
-                        const int h = (q >> 1) & 1, kb = (q & 1) | ((q >> 2) << 1);
-                        if (q == 0) {
-                            // inputs 0-127 written and accumulator half 0 drained
-                            if (!wait_abort(&h_ready[0], nh0 & 1u, abort, p.err, 12)) { ok = false; break; }
-                            ++nh0;
-                            tc_fence_after();
-                        }
-                        if (q == 2 && (L > 0 || t != blockIdx.x)) {
-                            // accumulator half 1 read by the previous half-1 epilogue
-                            if (!wait_abort(h1_drained, nd & 1u, abort, p.err, 19)) { ok = false; break; }
-                            ++nd;
-                            tc_fence_after();
-                        }
-                        if (q == 4) {
-                            // inputs 128-255 written
-                            if (!wait_abort(&h_ready[1], nh1 & 1u, abort, p.err, 13)) { ok = false; break; }
-                            ++nh1;
-                            tc_fence_after();
-                        }
-                        const uint32_t s = g % kStagesW;
-                        if (!wait_abort(&full[s], (g / kStagesW) & 1u, abort, p.err, 14)) { ok = false; break; }
-                        tc_fence_after();
-                        const uint32_t wb = smem_u32(sW + s * kChunkBytes);
+            for (int L = 0; L < 3 && ok; ++L) {
+                // order: half 0 over inputs 0-127, half 1 over inputs 0-127 (as soon as the
+                // previous half-1 epilogue has read its accumulator), half 0 over 128-255
+                // (once that epilogue has written them), half 1 over 128-255
+#pragma unroll 1
+                for (int q = 0; q < 8; ++q) {
+                    const int h = (q >> 1) & 1, kb = (q & 1) | ((q >> 2) << 1);
+                    // inputs 0-127 written and accumulator half 0 drained
+                    if (q == 0 && !wait(&h_ready[0], nh, 12)) { ok = false; break; }
+                    if (q == 2 && (L > 0 || t != blockIdx.x)) {
+                        // accumulator half 1 read by the previous half-1 epilogue
+                        if (!wait(h1_drained, nd, 19)) { ok = false; break; }
+                        ++nd;
+                    }
+                    // inputs 128-255 written
+                    if (q == 4 && !wait(&h_ready[1], nh, 13)) { ok = false; break; }
+                    if (!wait(&full[st], par, 14)) { ok = false; break; }
+                    if (leader) {
+                        const uint32_t a_lo = w_lo + st * (kChunkBytes / 16), b_lo = h_lo + kb * (4 * 8192 / 16);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tmem + h * 256, desc_sw128(wb + ks * 32),
-                                     desc_sw128_mn(hb + (kb * 4 + ks) * 8192, 1024, 4096), id_hid,
-                                     (kb | ks) ? 1u : 0u);
-                        mma_commit(&empty[s]);
-                        ++g;
+                            mma_bf16(tm + h * 256, desc_of(desc_hi(1024), a_lo + ks * (32 / 16)),
+                                     desc_of(desc_hi(4096), b_lo + ks * (8192 / 16)), id_hid, (uint32_t)(kb | ks));
+                        mma_commit(&empty[st]);
                         // half 0 complete, and with it every MMA of this layer over inputs 0-127
                         if (q == 5) mma_commit(&acc[0]);
+                        if (q == 7) mma_commit(&acc[1]);
                     }
-                    if (ok) mma_commit(&acc[1]);
+                    __syncwarp();
+                    if (++st == kStagesW) {
+                        st = 0;
+                        par ^= 1u;
+                    }
                 }
-                if (!ok) break;
-                // output layer: rows x W5^T, M-tile 0 into columns 0-15 and M-tile 1 into 16-31
-                // (both in the drained half-0 accumulator), in two K halves: input features
-                // 0-127 as soon as their epilogue is done, 128-255 after the last one
-                bool ok2 = true;
-                if (t == blockIdx.x) {
-                    // W5, loaded once per launch
-                    if (!wait_abort(w5full, 0, abort, p.err, 17)) break;
-                    tc_fence_after();
-                }
-                for (int kh = 0; kh < 2 && ok2; ++kh) {
-                    uint32_t &nh = kh ? nh1 : nh0;
-                    if (!wait_abort(&h_ready[kh], nh & 1u, abort, p.err, 15 + kh)) { ok2 = false; break; }
-                    ++nh;
-                    tc_fence_after();
-                    const uint32_t wb = smem_u32(sW5);
+                ++nh;
+            }
+            // output layer: rows x W5^T, M-tile 0 into columns 0-15 and M-tile 1 into 16-31
+            // (both in the drained half-0 accumulator), in two K halves: input features
+            // 0-127 as soon as their epilogue is done, 128-255 after the last one
+            for (int kh = 0; kh < 2 && ok; ++kh) {
+                if (!wait(&h_ready[kh], nh, 15 + kh)) { ok = false; break; }
+                if (leader) {
+                    const uint32_t w5_lo = desc_lo(smem_u32(sW5), 16);
 #pragma unroll
                     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
                         for (int k8 = 0; k8 < 8; ++k8) {
                             const int k16 = kh * 8 + k8;
-                            mma_bf16(tmem + mt * 16, desc_sw128_mn(hb + mt * 2048 + k16 * 8192, 1024, 4096),
-                                     desc_sw128(wb + (k16 >> 2) * 2048 + (k16 & 3) * 32), id_out, k16 ? 1u : 0u);
+                            mma_bf16(tm + mt * 16, desc_of(desc_hi(4096), h_lo + (mt * 2048 + k16 * 8192) / 16),
+                                     desc_of(desc_hi(1024), w5_lo + ((k16 >> 2) * 2048 + (k16 & 3) * 32) / 16), id_out,
+                                     k16 ? 1u : 0u);
                         }
-                    if (kh == 0) mma_commit(out_a);
+                    mma_commit(kh ? acc_out : out_a);
                 }
-                if (!ok2) break;
-                mma_commit(acc_out);
+                __syncwarp();
             }
-            // all MMAs of this CTA complete before its tensor memory is released
+            ++nh;
+        }
+        // all MMAs of this CTA complete before its tensor memory is released
+        if (leader) {
             mma_commit(fin);
             mbar_wait(fin, 0);
         }
+        __syncwarp();
     } else {
         // ------------------------------------------------------------ compute warps
         // warp w: tensor-memory lane quarter lq = w % 4 (features 32 lq .. of each half) and
