@@ -58,7 +58,7 @@ constexpr uint32_t kChunkBytes = 128u * 128u;   // 128 output rows x 64 bf16
 constexpr uint32_t kW5Bytes = 4u * 16u * 128u;  // W5 padded: 4 boxes of 16 rows x 64 bf16
 constexpr uint32_t kHBytes = 32u * 4u * 1024u;  // 32 K-groups x 4 MN-blocks of 1024 B
 constexpr int kChunksPerTile = 3 * 8;
-constexpr int kComputeThreads = 512;            // arrivals on each h_ready barrier
+constexpr int kComputeWarps = 16;               // arrivals on each h_ready barrier
 constexpr int kThreads = 576;
 constexpr int kMmaWarp = 16, kTmaWarp = 17;
 constexpr uint32_t kPtsBytes = 16u * 16u * 16u;  // per compute warp: its 16 points as float4
@@ -183,11 +183,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(&h_ready[0], kComputeThreads);
-        mbar_init(&h_ready[1], kComputeThreads);
+        mbar_init(&h_ready[0], kComputeWarps);
+        mbar_init(&h_ready[1], kComputeWarps);
         mbar_init(&acc[0], 1);
         mbar_init(&acc[1], 1);
-        mbar_init(h1_drained, kComputeThreads);
+        mbar_init(h1_drained, kComputeWarps);
         mbar_init(acc_out, 1);
         mbar_init(out_a, 1);
         mbar_init(fin, 1);
@@ -423,7 +423,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (rg < 2) tmem_ld16(lane_base + rg * 16, v);
                 }
                 tc_fence_before();
-                mbar_arrive(&h_ready[h]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&h_ready[h]);
                 if (h == 0 && !first && rg < 2)
                     store_out(p, b5, v, base_prev, rg * 128 + lq * 32 + lane, lane, n_pts);
             }
@@ -459,7 +460,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                             // the half-1 accumulator is read: the next layer's half-1 MMAs
                             // over inputs 0-127 may run during the rest of this epilogue
                             tc_fence_before();
-                            mbar_arrive(h1_drained);
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(h1_drained);
                         }
                         float o[4][8];
 #pragma unroll
@@ -482,7 +484,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(&h_ready[h]);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&h_ready[h]);
                 }
             }
             if (!ok) break;

@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&empty[s], 1);
         }
         for (int h = 0; h < 2; ++h) {
-            mbar_init(&h_ready[h], kComputeThreads);
+            mbar_init(&h_ready[h], kComputeThreads / 32);
             mbar_init(&acc[h], 1);
         }
         for (int r = 0; r < 4; ++r)
@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         auto announce = [&](int h) {
             fence_proxy_async_smem();
             tc_fence_before();
-            mbar_arrive(&h_ready[h]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&h_ready[h]);
         };
         for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
             const bool first = t == blockIdx.x;
