@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "gc_device.cuh"
 #include "gc_neural.h"
 #include "gc_siren.h"
 
@@ -80,48 +81,234 @@ __global__ void k_adam(float *__restrict__ P, float *__restrict__ G, float *__re
 // The eight channels of the trilinear grid interpolant at x (scaled by r_max), scaled as the
 // network's outputs. Same cell conventions as the push's gather: node-centred, poles
 // included, periodic in phi, clamped to the edge cells.
+struct TargetGeom {
+    int n_r, n_th, n_ph;
+    double r_min, dr, r_max, B_scale, E_scale;
+};
+
 template <typename T>
-__global__ void k_targets(const T *__restrict__ nodes, int n_r, int n_th, int n_ph, double r_min, double dr,
-                          const float *__restrict__ x, int64_t n, double r_max, double B_scale, double E_scale,
+__device__ __forceinline__ void target_point(const T *__restrict__ nodes, const TargetGeom &g, float x, float y, float z,
+                                             float *__restrict__ out)
+{
+    const double X = (double)x * g.r_max, Y = (double)y * g.r_max, Zc = (double)z * g.r_max;
+    const double rho = sqrt(X * X + Y * Y), r = sqrt(X * X + Y * Y + Zc * Zc);
+    const double th = atan2(rho, Zc);
+    double ph = atan2(Y, X);
+    if (ph < 0) ph += 2.0 * kPi;
+    const double xr = (r - g.r_min) / g.dr, xt = th / (kPi / (g.n_th - 1)), xp = ph / (2.0 * kPi / g.n_ph);
+    int i = (int)floor(xr);
+    double fr = xr - i;
+    if (i < 0) { i = 0; fr = 0; }
+    else if (i > g.n_r - 2) { i = g.n_r - 2; fr = 1; }
+    int j = (int)floor(xt);
+    double ft = xt - j;
+    if (j < 0) { j = 0; ft = 0; }
+    else if (j > g.n_th - 2) { j = g.n_th - 2; ft = 1; }
+    int k = (int)floor(xp);
+    const double fp = xp - k;
+    if (k >= g.n_ph) k -= g.n_ph;
+    if (k < 0) k += g.n_ph;
+    const int k1 = (k + 1 == g.n_ph) ? 0 : k + 1;
+    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 2; ++b)
+            for (int c = 0; c < 2; ++c) {
+                const double w = (a ? fr : 1 - fr) * (b ? ft : 1 - ft) * (c ? fp : 1 - fp);
+                const T *p = nodes + (((int64_t)(c ? k1 : k) * g.n_th + (j + b)) * g.n_r + (i + a)) * 8;
+                for (int ch = 0; ch < 8; ++ch)
+                    v[ch] += w * (double)p[ch];
+            }
+    const double a1 = r / kAU;
+    const double sb = a1 * a1 / g.B_scale, se = a1 / g.E_scale;
+    for (int ch = 0; ch < 3; ++ch) {
+        out[ch] = (float)(v[ch] * sb);
+        out[3 + ch] = (float)(v[3 + ch] * se);
+    }
+    out[6] = (float)(v[6] * sb);
+    out[7] = (float)(v[7] / (g.E_scale * kAU));
+}
+
+template <typename T>
+__global__ void k_targets(const T *__restrict__ nodes, const TargetGeom g, const float *__restrict__ x, int64_t n,
                           float *__restrict__ out)
 {
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
+        target_point(nodes, g, x[3 * q], x[3 * q + 1], x[3 * q + 2], out + 8 * q);
+}
+
+// The same from an FP32 grid, in pairs of floats (value hi + lo, about 2^-45): GB300 runs
+// FP64 at 1/64 of FP32, and a point takes some 500 FP64 operations and conversions above.
+// Error-free sums and products (Dekker 1971, Knuth) carry every step below, so the result is
+// the float nearest the FP64 one but for about one value in 10^5. 2^20 points of the 256 x 128
+// x 256 grid: 688 us in FP64, 70 us so (the 8 corner records, at random, are 270 MB).
+struct ff {
+    float h, l;
+};
+__host__ __device__ inline ff ff_of(double d)
+{
+    const float h = (float)d;
+    return {h, (float)(d - (double)h)};
+}
+__device__ __forceinline__ ff ff_norm(float h, float l) // |h| >= |l|
+{
+    const float s = __fadd_rn(h, l);
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ ff ff_sum(float a, float b) // a + b exactly
+{
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ ff ff_prod(float a, float b) // a b exactly
+{
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ ff ff_add(ff a, ff b)
+{
+    const ff s = ff_sum(a.h, b.h);
+    return ff_norm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ ff ff_mul(ff a, ff b)
+{
+    const ff p = ff_prod(a.h, b.h);
+    return ff_norm(p.h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, p.l)));
+}
+__device__ __forceinline__ ff ff_mul(ff a, float b)
+{
+    const ff p = ff_prod(a.h, b);
+    return ff_norm(p.h, __fmaf_rn(a.l, b, p.l));
+}
+// 1 / sqrt(a): one Newton step on the float estimate (relative error e < 2^-21 -> 3/8 e^2)
+__device__ __forceinline__ ff ff_rsqrt(ff a)
+{
+    const float y = rsqrtf(a.h);
+    const ff u = ff_mul(a, ff_prod(y, y));
+    return ff_norm(y, __fmul_rn(__fmul_rn(0.5f, y), __fsub_rn(__fsub_rn(1.0f, u.h), u.l)));
+}
+
+// Index coordinate angle / step of the polar angle of (X, Y), given 1 / hypot(X, Y): the offset
+// from the nearest of 256 tabulated angles by the arcsine's series, as in the push's FP64
+// path (refine_angle); k256 = 2 pi / 256 / step, inv = 1 / step.
+__device__ __forceinline__ ff ff_angle(ff X, ff Y, ff inv_h, const float4 *table, ff k256, ff inv)
+{
+    const int m = __float2int_rn(gcp::m_atan2(Y.h, X.h) * (float)kCircleInvStep) & (GC_CIRCLE_N - 1);
+    const float4 cs = table[m];
+    const ff yc = ff_mul(Y, ff{cs.x, cs.y}), xs = ff_mul(X, ff{cs.z, cs.w});
+    const ff t = ff_mul(ff_add(yc, ff{-xs.h, -xs.l}), inv_h);
+    const float t2 = t.h * t.h;
+    const float p = fmaf(fmaf(t2, 5.0f / 112.0f, 3.0f / 40.0f), t2, 1.0f / 6.0f);
+    const ff d = ff_norm(t.h, __fmaf_rn(t.h * t2, p, t.l));
+    return ff_add(ff_mul(k256, (float)m), ff_mul(d, inv));
+}
+
+// cell index and fraction in [0, 1] of an index coordinate
+__device__ __forceinline__ int ff_cell(ff x, ff &f)
+{
+    float fl = floorf(x.h);
+    f = ff_norm(__fsub_rn(x.h, fl), x.l);
+    if (f.h < 0.f) { // x.h whole, x.l negative
+        fl -= 1.f;
+        f = ff_norm(1.f, f.h);
+    }
+    return (int)fl;
+}
+
+struct TargetGeomF {
+    ff rr, r0, kt, it, kp, ip; // r_max / dr, r_min / dr; 2 pi / 256 and 1 in units of the theta, phi steps
+    ff au, ib, ie, ip7;        // r_max / AU, 1 / B_scale, 1 / E_scale, 1 / (E_scale AU)
+};
+
+__device__ __noinline__ void target_point_f64(const float *nodes, const TargetGeom &g, float x, float y, float z, float *out)
+{
+    target_point(nodes, g, x, y, z, out);
+}
+
+__global__ void __launch_bounds__(128) k_targets_ff(const float *__restrict__ nodes, const __grid_constant__ TargetGeom g,
+                                                    const __grid_constant__ TargetGeomF G, const float *__restrict__ x,
+                                                    int64_t n, float *__restrict__ out)
+{
+    __shared__ float4 table[GC_CIRCLE_N]; // cos and sin of the reference angles as pairs
+    for (int m = threadIdx.x; m < GC_CIRCLE_N; m += blockDim.x) {
+        const double2 cs = kUnitCircle[m];
+        const ff c = ff_of(cs.x), s = ff_of(cs.y);
+        table[m] = make_float4(c.h, c.l, s.h, s.l);
+    }
+    __syncthreads();
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        const double X = (double)x[3 * q] * r_max, Y = (double)x[3 * q + 1] * r_max, Zc = (double)x[3 * q + 2] * r_max;
-        const double rho = sqrt(X * X + Y * Y), r = sqrt(X * X + Y * Y + Zc * Zc);
-        const double th = atan2(rho, Zc);
-        double ph = atan2(Y, X);
-        if (ph < 0) ph += 2.0 * kPi;
-        const double xr = (r - r_min) / dr, xt = th / (kPi / (n_th - 1)), xp = ph / (2.0 * kPi / n_ph);
-        int i = (int)floor(xr);
-        double fr = xr - i;
-        if (i < 0) { i = 0; fr = 0; }
-        else if (i > n_r - 2) { i = n_r - 2; fr = 1; }
-        int j = (int)floor(xt);
-        double ft = xt - j;
-        if (j < 0) { j = 0; ft = 0; }
-        else if (j > n_th - 2) { j = n_th - 2; ft = 1; }
-        int k = (int)floor(xp);
-        const double fp = xp - k;
-        if (k >= n_ph) k -= n_ph;
-        if (k < 0) k += n_ph;
-        const int k1 = (k + 1 == n_ph) ? 0 : k + 1;
-        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b)
-                for (int c = 0; c < 2; ++c) {
-                    const double w = (a ? fr : 1 - fr) * (b ? ft : 1 - ft) * (c ? fp : 1 - fp);
-                    const T *p = nodes + (((int64_t)(c ? k1 : k) * n_th + (j + b)) * n_r + (i + a)) * 8;
-                    for (int ch = 0; ch < 8; ++ch)
-                        v[ch] += w * (double)p[ch];
+        const float X = x[3 * q], Y = x[3 * q + 1], Z = x[3 * q + 2];
+        const ff rho2 = ff_add(ff_prod(X, X), ff_prod(Y, Y)), r2 = ff_add(rho2, ff_prod(Z, Z));
+        float o[8];
+        // pairs lose their low words near the limits of the format (and on the axis): FP64 there
+        bool ok = rho2.h > 1e-20f && r2.h < 1e20f;
+        if (ok) {
+            const ff ir = ff_rsqrt(r2), irho = ff_rsqrt(rho2);
+            const ff r = ff_mul(r2, ir), rho = ff_mul(rho2, irho);
+            const ff b0 = ff_mul(r, G.rr);
+            const ff xr = ff_add(b0, ff{-G.r0.h, -G.r0.l});
+            const ff xt = ff_angle(ff{Z, 0.f}, rho, ir, table, G.kt, G.it);
+            ff xp = ff_angle(ff{X, 0.f}, ff{Y, 0.f}, irho, table, G.kp, G.ip);
+            if (xp.h < 0.f) xp = ff_add(xp, ff{(float)g.n_ph, 0.f});
+            ff fr, ft, fp;
+            int i = xr.h < -1.f ? -1 : (xr.h > (float)g.n_r ? g.n_r : ff_cell(xr, fr));
+            int j = ff_cell(xt, ft), k = ff_cell(xp, fp);
+            if (i < 0) { i = 0; fr = ff{0.f, 0.f}; }
+            else if (i > g.n_r - 2) { i = g.n_r - 2; fr = ff{1.f, 0.f}; }
+            if (j < 0) { j = 0; ft = ff{0.f, 0.f}; }
+            else if (j > g.n_th - 2) { j = g.n_th - 2; ft = ff{1.f, 0.f}; }
+            if (k >= g.n_ph) k -= g.n_ph;
+            if (k < 0) k += g.n_ph;
+            const int k1 = (k + 1 == g.n_ph) ? 0 : k + 1;
+            const ff gr = ff_add(ff{1.f, 0.f}, ff{-fr.h, -fr.l}), gt = ff_add(ff{1.f, 0.f}, ff{-ft.h, -ft.l}),
+                     gp = ff_add(ff{1.f, 0.f}, ff{-fp.h, -fp.l});
+            float vh[8], vl[8];
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch)
+                vh[ch] = vl[ch] = 0.f;
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const ff wtp = ff_mul(b ? ft : gt, c ? fp : gp);
+                    const float4 *p = reinterpret_cast<const float4 *>(
+                        nodes + (((int64_t)(c ? k1 : k) * g.n_th + (j + b)) * g.n_r + i) * 8);
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        const ff w = ff_mul(a ? fr : gr, wtp);
+                        const float4 pa = __ldg(p + 2 * a), pb = __ldg(p + 2 * a + 1);
+                        const float pv[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+#pragma unroll
+                        for (int ch = 0; ch < 8; ++ch) {
+                            const ff t = ff_prod(pv[ch], w.h);
+                            const ff s = ff_sum(vh[ch], t.h);
+                            vh[ch] = s.h;
+                            vl[ch] = __fadd_rn(vl[ch], __fadd_rn(s.l, __fmaf_rn(pv[ch], w.l, t.l)));
+                        }
+                    }
                 }
-        const double a1 = r / kAU;
-        const double sb = a1 * a1 / B_scale, se = a1 / E_scale;
-        for (int ch = 0; ch < 3; ++ch) {
-            out[8 * q + ch] = (float)(v[ch] * sb);
-            out[8 * q + 3 + ch] = (float)(v[3 + ch] * se);
+            const ff a1 = ff_mul(r, G.au);
+            const ff sb = ff_mul(ff_mul(a1, a1), G.ib), se = ff_mul(a1, G.ie);
+            ok = sb.h > 1e-20f && sb.h < 1e20f && se.h > 1e-20f && se.h < 1e20f && G.ip7.h > 1e-20f && G.ip7.h < 1e20f;
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch) {
+                const float a = fabsf(vh[ch]);
+                // zero, or in the range where the low words are normal (a NaN fails)
+                ok = ok && (a == 0.f || (a > 1e-18f && a < 1e18f));
+                const ff sc = ch < 3 || ch == 6 ? sb : (ch == 7 ? G.ip7 : se);
+                const ff t = ff_prod(vh[ch], sc.h);
+                o[ch] = __fadd_rn(t.h, __fmaf_rn(vl[ch], sc.h, __fmaf_rn(vh[ch], sc.l, t.l)));
+            }
         }
-        out[8 * q + 6] = (float)(v[6] * sb);
-        out[8 * q + 7] = (float)(v[7] / (E_scale * kAU));
+        if (!ok) target_point_f64(nodes, g, X, Y, Z, o);
+        float4 *dst = reinterpret_cast<float4 *>(out + 8 * q);
+        if (((uintptr_t)out & 15u) == 0) {
+            dst[0] = make_float4(o[0], o[1], o[2], o[3]);
+            dst[1] = make_float4(o[4], o[5], o[6], o[7]);
+        } else {
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch)
+                out[8 * q + ch] = o[ch];
+        }
     }
 }
 
@@ -240,16 +427,20 @@ cudaError_t neural_field_at(Neural &nn, const float *R, int64_t cap, const int32
     return gcs::siren_eval(nn.net, in, o, s);
 }
 
-cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, int64_t n, float *t, cudaStream_t s)
+cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, int64_t n, float *out, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int b = blocks_for(n, 128);
-    if (g.is_f64)
-        k_targets<double><<<b, 128, 0, s>>>((const double *)g.nodes, g.n_r, g.n_th, g.n_ph, g.r_min, g.dr, x, n,
-                                            nn.r_max, nn.B_scale, nn.E_scale, t);
-    else
-        k_targets<float><<<b, 128, 0, s>>>((const float *)g.nodes, g.n_r, g.n_th, g.n_ph, g.r_min, g.dr, x, n,
-                                           nn.r_max, nn.B_scale, nn.E_scale, t);
+    const TargetGeom t{g.n_r, g.n_th, g.n_ph, g.r_min, g.dr, nn.r_max, nn.B_scale, nn.E_scale};
+    if (g.is_f64) {
+        k_targets<double><<<b, 128, 0, s>>>((const double *)g.nodes, t, x, n, out);
+    } else {
+        const double it = (g.n_th - 1) / kPi, ip = g.n_ph / (2.0 * kPi);
+        const TargetGeomF f{ff_of(nn.r_max / g.dr), ff_of(g.r_min / g.dr), ff_of(kCircleStep * it), ff_of(it),
+                            ff_of(kCircleStep * ip), ff_of(ip), ff_of(nn.r_max / kAU), ff_of(1.0 / nn.B_scale),
+                            ff_of(1.0 / nn.E_scale), ff_of(1.0 / (nn.E_scale * kAU))};
+        k_targets_ff<<<b, 128, 0, s>>>((const float *)g.nodes, t, f, x, n, out);
+    }
     return cudaGetLastError();
 }
 

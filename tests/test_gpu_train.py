@@ -37,3 +37,39 @@ def test_gradient_at_tile_edges(n, omega0, tol):
         err = np.linalg.norm(g[k] - go[k]) / np.linalg.norm(go[k])
         print(k, err)
         assert err < 5 * tol, k
+
+
+def test_targets_are_the_rounded_interpolant():
+    """Training targets from an FP32 grid (pairs of floats; FP64 where those end) against the
+    FP64 interpolant: within a float's rounding (2^-24) of each value, plus 1e-10 of the
+    channel's scale for index coordinates that agree to 1e-11. Points inside, across the cell
+    faces, at the poles and on the axis, at phi = 0, outside the shell on both sides, and so
+    near the origin that pairs would underflow; scales at both ends of what pairs hold."""
+    w = synth.WindSpec(33, 17, 21, eps=0.1, n_modes=4, phi1_v=100.0)
+    nodes = synth.wind_grid(w, dtype=np.float32)
+    rng = np.random.default_rng(3)
+    x = rng.normal(size=(20000, 3))
+    x *= (rng.uniform(0.02, 1.2, (len(x), 1)) / np.linalg.norm(x, axis=1, keepdims=True))
+    r = (w.r_min_au + w.dr_au * rng.integers(0, w.n_r, 4000)) / w.r_max_au
+    th = np.pi * rng.integers(0, w.n_th, 4000) / (w.n_th - 1)
+    ph = 2 * np.pi * rng.integers(0, w.n_ph, 4000) / w.n_ph
+    node = np.stack([r * np.sin(th) * np.cos(ph), r * np.sin(th) * np.sin(ph), r * np.cos(th)], 1)
+    special = np.array([[0, 0, 0.5], [0, 0, -0.5], [0.5, 0, 0], [-0.5, 0, 0], [0.5, -0.0, 0.1], [1e-15, 0, 0.4],
+                        [1e-30, 1e-30, 1e-30], [0.3, -1e-20, 0.2], [3, 2, 1], [1e-3, 1e-3, 1e-3]])
+    x = np.concatenate([x, node, special]).astype(np.float32)
+    for B_s, E_s in ((3.5e-9, 1.4e-3), (1e-25, 1.4e-3), (3.5e-9, 1e22)):
+        with gcpush.Context() as c:
+            c.field_load(nodes, w.r_min_au, w.r_max_au)
+            c.siren_set(synth.siren_init(0), r_max_au=w.r_max_au, B_scale=B_s, E_scale=E_s)
+            t = torch.full((len(x), 8), float("nan"), device="cuda")
+            c.field_targets(torch.from_numpy(x).cuda(), t)
+            odd = torch.full((8 * len(x) + 1,), float("nan"), device="cuda")  # output at 4-byte alignment
+            c.field_targets(torch.from_numpy(x).cuda(), odd[1:].view(-1, 8))
+        t = t.cpu().numpy()
+        assert np.array_equal(t, odd[1:].cpu().numpy().reshape(-1, 8))
+        to = siren.grid_targets(nodes.astype(np.float64), w.r_min_au * siren.AU, w.r_max_au * siren.AU,
+                                x.astype(np.float64), w.r_max_au * siren.AU, B_s, E_s)
+        scale = np.sqrt((to * to).mean(0))
+        err = np.abs(t - to) / (2.0**-24 * np.abs(to) * 1.0001 + 1e-10 * scale + 1e-45)
+        print(err.max(0))
+        assert err.max() <= 1.0
