@@ -181,7 +181,7 @@ struct gc_ctx {
     double field_ms = 0.0;
 
     // launch shape
-    int block = 128;
+    int block = 0;           // 0: see push_block
     int grid_waves = 1;      // resident waves of blocks (0: one thread per particle)
     int blocks_per_sm[5] = {0, 0, 0, 0, 0}; // occupancy per block size / 32, cached
     int steps_per_launch = 2000;
@@ -365,16 +365,32 @@ int do_sort(gc_ctx *c, cudaStream_t s, std::vector<Timed> *owned, LaunchCounts *
     return GC_OK;
 }
 
-int push_grid(gc_ctx *c)
+int blocks_per_sm(gc_ctx *c, int block)
 {
-    int &nb = c->blocks_per_sm[c->block / 32];
+    int &nb = c->blocks_per_sm[block / 32];
     if (nb <= 0) {
-        nb = gcp::push_max_blocks_per_sm(c->opt.precision, c->block, c->gh.nodes1 != nullptr,
-                                        c->gh.ideal == 2);
+        nb = gcp::push_max_blocks_per_sm(c->opt.precision, block, c->gh.nodes1 != nullptr, c->gh.ideal == 2);
         cudaGetLastError(); // an occupancy query failure only means "one block"
         if (nb < 1) nb = 1;
     }
-    const int64_t want = (c->n + c->block - 1) / c->block;
+    return nb;
+}
+
+// Threads per block of the push: what gc_set_launch or the autotuner chose, else 32 while one
+// resident wave holds all particles (warps then spread evenly over the SMs: FP32 of 40 000
+// particles 1.78e10 -> 1.88e10 particle-steps/s, FP64 of 4096 / 30 000 1.43e8 -> 1.54e8 /
+// 5.4e8 -> 6.1e8) and 128 beyond (neighbouring groups of particles, which share cells, on one
+// SM: 64 ensembles at as many sites run 23 % slower with 32).
+int push_block(gc_ctx *c)
+{
+    if (c->block) return c->block;
+    return c->n <= (int64_t)c->sm_count * blocks_per_sm(c, 128) * 128 ? 32 : 128;
+}
+
+int push_grid(gc_ctx *c, int block)
+{
+    const int nb = blocks_per_sm(c, block);
+    const int64_t want = (c->n + block - 1) / block;
     if (c->grid_waves <= 0)
         return (int)std::min<int64_t>(want, 0x7FFFFFFF);
     return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)c->grid_waves * c->sm_count * nb));
@@ -386,7 +402,7 @@ int push_grid(gc_ctx *c)
 int enqueue_advance(gc_ctx *c, cudaStream_t s, double dt, int64_t n_steps, double lambda_au,
                     const double *clock_dev, std::vector<Timed> *owned, LaunchCounts *lc)
 {
-    const int grid = push_grid(c);
+    const int block = push_block(c), grid = push_grid(c, block);
     gcp::PushParams P{};
     P.st = c->st;
     P.ens = c->d_ens;
@@ -424,7 +440,7 @@ int enqueue_advance(gc_ctx *c, cudaStream_t s, double dt, int64_t n_steps, doubl
         Timed t;
         TRY(new_interval(c, 0, owned, &t));
         CUDA_TRY(cudaEventRecord(t.a, s));
-        CUDA_TRY(gcp::launch_push(c->opt.precision, c->gh, ph, P, c->block, grid, s));
+        CUDA_TRY(gcp::launch_push(c->opt.precision, c->gh, ph, P, block, grid, s));
         CUDA_TRY(cudaEventRecord(t.b, s));
         lc->kernels += 1;
         lc->pushes += 1;
@@ -505,7 +521,7 @@ int advance_graph(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool 
         }
         CUDA_TRY(gcp::preload_kernels());
         CUDA_TRY(gcp::sort_preload());
-        push_grid(c); // occupancy query outside the capture
+        push_grid(c, push_block(c)); // occupancy queries outside the capture
         CUDA_TRY(cudaStreamSynchronize(c->stream));
         cudaGetLastError(); // start the capture with no stale error
         G = new GraphEntry();
