@@ -175,8 +175,9 @@ struct gc_ctx {
 
     // split-step push buffers (sources other than the inline grid gather)
     int64_t split_cap = 0;
-    float *d_req = nullptr, *d_reqR = nullptr, *d_S = nullptr, *d_SR = nullptr;
-    int32_t *d_list = nullptr, *d_count = nullptr;
+    float *d_req = nullptr, *d_S = nullptr;
+    int32_t *d_prog = nullptr, *d_list[2] = {nullptr, nullptr}, *d_count = nullptr; // d_count: [2]
+    int32_t *h_count = nullptr; // pinned
     uint64_t field_evals = 0;
     double field_ms = 0.0;
 
@@ -604,11 +605,12 @@ int advance_graph(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool 
 // and for the grid evaluated through the same sample buffers (GC_FIELD_GRID_SAMPLED).
 void free_split(gc_ctx *c)
 {
-    void *p[] = {c->d_req, c->d_reqR, c->d_S, c->d_SR, c->d_list, c->d_count};
+    void *p[] = {c->d_req, c->d_S, c->d_prog, c->d_list[0], c->d_list[1], c->d_count};
     for (void *q : p)
         if (q) cudaFree(q);
-    c->d_req = c->d_reqR = c->d_S = c->d_SR = nullptr;
-    c->d_list = c->d_count = nullptr;
+    if (c->h_count) cudaFreeHost(c->h_count);
+    c->d_req = c->d_S = nullptr;
+    c->d_prog = c->d_list[0] = c->d_list[1] = c->d_count = c->h_count = nullptr;
     c->split_cap = 0;
 }
 
@@ -618,11 +620,12 @@ int ensure_split(gc_ctx *c)
     free_split(c);
     const size_t n = (size_t)std::max<int64_t>(c->cap, 1);
     CUDA_TRY(cudaMalloc(&c->d_req, n * 3 * sizeof(float)));
-    CUDA_TRY(cudaMalloc(&c->d_reqR, n * 3 * sizeof(float)));
     CUDA_TRY(cudaMalloc(&c->d_S, n * gcp::kSampleStride * sizeof(float)));
-    CUDA_TRY(cudaMalloc(&c->d_SR, n * gcp::kSampleStride * sizeof(float)));
-    CUDA_TRY(cudaMalloc(&c->d_list, n * sizeof(int32_t)));
-    CUDA_TRY(cudaMalloc(&c->d_count, sizeof(int32_t)));
+    CUDA_TRY(cudaMalloc(&c->d_prog, n * sizeof(int32_t)));
+    for (int32_t *&l : c->d_list)
+        CUDA_TRY(cudaMalloc(&l, n * sizeof(int32_t)));
+    CUDA_TRY(cudaMallocHost(&c->h_count, sizeof(int32_t)));
+    CUDA_TRY(cudaMalloc(&c->d_count, 2 * sizeof(int32_t)));
     c->split_cap = (int64_t)n;
     return GC_OK;
 }
@@ -666,17 +669,14 @@ gcp::SplitParams split_params(gc_ctx *c, double dt, double lambda_au)
     P.counters = c->d_counters;
     Q.req = c->d_req;
     Q.S = c->d_S;
-    Q.reqR = c->d_reqR;
-    Q.SR = c->d_SR;
-    Q.list = c->d_list;
-    Q.count = c->d_count;
+    Q.prog = c->d_prog;
     Q.g_in_sample = c->field_source == GC_FIELD_SIREN ? 0 : 1;
     Q.ideal = c->gh.ideal;
     return Q;
 }
 
-// n_steps steps of the split-step push: per step the predictor requests, two evaluations
-// of all particles, and two evaluations of the restart list
+// n_steps steps of the split-step push: two rounds per step over all particles, then rounds
+// over the list of those that rebirths and collisions held up
 int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool *anomaly)
 {
     TRY(ensure_split(c));
@@ -685,20 +685,41 @@ int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool 
     cudaStream_t s = c->stream;
     LaunchCounts lc;
     const uint64_t coll0 = c->collisions, reb0 = c->rebirths;
-    for (int64_t k = 0; k < n_steps; ++k) {
-        Q.kk = (long long)(k + 1);
-        Q.tally_now = (c->tally_on && ((c->step + k + 1) % c->tdev.cadence == 0)) ? 1 : 0;
-        CUDA_TRY(cudaMemsetAsync(c->d_count, 0, sizeof(int32_t), s));
-        CUDA_TRY(gcp::launch_split(gcp::SPLIT_PRED, ph, Q, s));
-        TRY(field_samples(c, c->d_req, c->n, nullptr, c->d_S, &lc));
-        CUDA_TRY(gcp::launch_split(gcp::SPLIT_CORR, ph, Q, s));
-        TRY(field_samples(c, c->d_req, c->n, nullptr, c->d_S, &lc));
-        CUDA_TRY(gcp::launch_split(gcp::SPLIT_POST, ph, Q, s));
-        TRY(field_samples(c, c->d_reqR, c->n, c->d_count, c->d_SR, &lc));
-        CUDA_TRY(gcp::launch_split(gcp::SPLIT_R2, ph, Q, s));
-        TRY(field_samples(c, c->d_reqR, c->n, c->d_count, c->d_SR, &lc));
-        CUDA_TRY(gcp::launch_split(gcp::SPLIT_R3, ph, Q, s));
-        lc.kernels += 5;
+    Q.P.step0 = c->step;
+    for (int64_t done = 0; done < n_steps; done += Q.P.n_steps) {
+        Q.P.n_steps = (int32_t)std::min<int64_t>(n_steps - done, 1 << 20);
+        Q.kbase = done;
+        Q.list_in = Q.count_in = nullptr;
+        Q.list_out = Q.count_out = nullptr;
+        CUDA_TRY(cudaMemsetAsync(c->d_count, 0, 2 * sizeof(int32_t), s));
+        CUDA_TRY(gcp::launch_split(gcp::SPLIT_INIT, ph, Q, c->n, s));
+        lc.kernels += 1;
+        for (int64_t r = 2 * (int64_t)Q.P.n_steps; r > 0; --r) {
+            TRY(field_samples(c, c->d_req, c->n, nullptr, c->d_S, &lc));
+            if (r == 1) { // the particles not done go into a list
+                Q.list_out = c->d_list[0];
+                Q.count_out = c->d_count;
+            }
+            CUDA_TRY(gcp::launch_split(gcp::SPLIT_ROUND, ph, Q, c->n, s));
+            lc.kernels += 1;
+        }
+        for (int cur = 0;;) {
+            CUDA_TRY(cudaMemcpyAsync(c->h_count, c->d_count + cur, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            CUDA_TRY(cudaStreamSynchronize(s));
+            const int64_t left = *c->h_count;
+            if (left == 0) break;
+            // a restart takes two rounds more; the count is looked at after each two
+            for (int r = 0; r < 2; ++r, cur ^= 1) {
+                TRY(field_samples(c, c->d_req, left, c->d_count + cur, c->d_S, &lc));
+                Q.list_in = c->d_list[cur];
+                Q.count_in = c->d_count + cur;
+                Q.list_out = c->d_list[cur ^ 1];
+                Q.count_out = c->d_count + (cur ^ 1);
+                CUDA_TRY(cudaMemsetAsync(Q.count_out, 0, sizeof(int32_t), s));
+                CUDA_TRY(gcp::launch_split(gcp::SPLIT_ROUND, ph, Q, left, s));
+                lc.kernels += 1;
+            }
+        }
     }
     add_counts(c, lc);
     TRY(collect_status(c, anomaly));
@@ -717,14 +738,11 @@ int split_inject_fix(gc_ctx *c, int64_t slot0, int64_t n_new)
     const gcp::PhysHost ph = c->phys();
     cudaStream_t s = c->stream;
     LaunchCounts lc;
-    const int32_t cnt = (int32_t)n_new;
-    CUDA_TRY(gcp::launch_split(gcp::SPLIT_INJ_REQ, ph, Q, s));
+    CUDA_TRY(gcp::launch_split(gcp::SPLIT_INJ_REQ, ph, Q, n_new, s));
     TRY(field_samples(c, c->d_req, n_new, nullptr, c->d_S, &lc));
-    CUDA_TRY(gcp::launch_split(gcp::SPLIT_INJ_FIX, ph, Q, s));
-    CUDA_TRY(cudaMemcpyAsync(c->d_count, &cnt, sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    TRY(field_samples(c, c->d_reqR, n_new, c->d_count, c->d_SR, &lc));
-    CUDA_TRY(gcp::launch_split(gcp::SPLIT_R3, ph, Q, s));
-    CUDA_TRY(cudaStreamSynchronize(s)); // the host word cnt is read by the copy above
+    CUDA_TRY(gcp::launch_split(gcp::SPLIT_INJ_FIX, ph, Q, n_new, s));
+    TRY(field_samples(c, c->d_req, n_new, nullptr, c->d_S, &lc));
+    CUDA_TRY(gcp::launch_split(gcp::SPLIT_INJ_FIN, ph, Q, n_new, s));
     lc.kernels += 3;
     add_counts(c, lc);
     c->field_evals += (uint64_t)(2 * n_new);

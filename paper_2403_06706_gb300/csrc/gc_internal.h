@@ -71,26 +71,25 @@ struct InjectParams {
 };
 
 // Split-step push: the state machine of the fused push cut at each field evaluation, for
-// field sources that evaluate many points at once (the neural field). Per step:
-//   PRED (all) -> samples -> CORR (all) -> samples -> POST (all; restarts join a list)
-//   -> samples (list) -> R2 (list) -> samples (list) -> R3 (list).
-// INJ_REQ / INJ_FIX redo the field-dependent part of the injection with the samples.
+// field sources that evaluate many points at once (the neural field):
+//   INIT -> samples -> ROUND -> samples -> ROUND ..
+// A round consumes one sample per unfinished particle, each in its own phase, and leaves the
+// next request; the rounds of the last particles run on a compact list.
+// INJ_REQ / INJ_FIX / INJ_FIN redo the field-dependent part of the injection with the samples.
 constexpr int kSampleStride = 40; // B, E, dB, dE (24), g (9), flags (1), dPhi (3), pad (3)
-enum SplitKind { SPLIT_PRED = 0, SPLIT_CORR, SPLIT_POST, SPLIT_R2, SPLIT_R3, SPLIT_INJ_REQ, SPLIT_INJ_FIX };
+enum SplitKind { SPLIT_INIT = 0, SPLIT_ROUND, SPLIT_INJ_REQ, SPLIT_INJ_FIX, SPLIT_INJ_FIN };
 
 struct SplitParams {
-    PushParams P;          // state, ensembles, physics switches, tallies, counters; P.dt, P.t0
-    float *req;            // [cap][3] request points (m), one per particle slot
+    PushParams P;          // state, ensembles, physics switches, tallies, counters; P.dt, P.t0,
+                           // P.step0 (the call's first step), P.n_steps (of these rounds)
+    float *req;            // [cap][3] request points (m): one per particle slot or list entry
     const float *S;        // [cap][kSampleStride] field samples at req
-    float *reqR;           // [cap][3] requests of the restart list
-    const float *SR;       // samples at reqR
-    int32_t *list;         // slots of the restart list
-    int32_t *count;        // entries in the list (device)
+    int32_t *prog;         // [cap] progress of each particle within these rounds
+    const int32_t *list_in, *count_in; // particles of this round (null: all)
+    int32_t *list_out, *count_out;     // list of the unfinished for the next round (null: in place)
     int32_t g_in_sample;   // 1: index-space derivatives and g in the sample (grid), 0: Cartesian
-    int32_t tally_now;     // this step ends on a tally sample
     int32_t ideal;         // drop E_par (ideal MHD field)
-    int32_t pad;
-    long long kk;          // t_new = t0 + kk dt for this step
+    long long kbase;       // steps of the call before these rounds
     int64_t slot0, n_new;  // injection fix-up: slots [slot0, slot0 + n_new)
 };
 
@@ -115,8 +114,8 @@ cudaError_t launch_push(int precision, const GridHost &g, const PhysHost &ph, co
 cudaError_t launch_inject(int precision, const GridHost &g, const PhysHost &ph,
                           const InjectParams &p, cudaStream_t s);
 int push_max_blocks_per_sm(int precision, int block, bool time_dependent = false, bool potential = false);
-// one split-step kernel (FP32 path)
-cudaError_t launch_split(int kind, const PhysHost &ph, const SplitParams &p, cudaStream_t s);
+// one split-step kernel (FP32 path) over n particles or list entries (at most)
+cudaError_t launch_split(int kind, const PhysHost &ph, const SplitParams &p, int64_t n, cudaStream_t s);
 // grid field samples (FP32 grid) at R (cap x 3, m; count on the device or cap)
 cudaError_t launch_grid_samples(const GridHost &g, const float *R, int64_t cap, const int32_t *n_dev, float *S,
                                 cudaStream_t s);

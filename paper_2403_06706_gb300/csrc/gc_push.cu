@@ -825,8 +825,15 @@ __global__ void __launch_bounds__(256) inject_kernel(const GridMeta<T> gm, const
 }
 
 // ----------------------------------------------------------------------------------------
-// Split-step push (FP32 path). Each kernel advances every particle (or every entry of the
-// restart list) by one evaluation phase, using the field samples of its request points.
+// Split-step push (FP32 path): the step cut at its field evaluations, for sources that
+// evaluate many points at once. Every particle walks the phases above at its own pace: a round
+// consumes one field sample per unfinished particle and asks for the next one, so the two
+// evaluations of a restart after a collision or rebirth are part of the rounds that the
+// other particles' next step needs anyway, and a particle is behind by a step per event. After
+// 2 n_steps rounds the few particles still behind go on in a compact list.
+// (With PRED, CORR, POST and two restart kernels and four evaluations per step, in lockstep,
+// 1024 particles took 97 us per step: each evaluation has a latency of about 16 us whatever the
+// number of points.)
 __device__ __forceinline__ void load_sample(const float *__restrict__ S, int64_t k, int g_in, Sample<float> &s)
 {
     const float4 *q = reinterpret_cast<const float4 *>(S + k * kSampleStride);
@@ -874,6 +881,25 @@ __device__ __forceinline__ void flush_counters(const PushParams &P, unsigned n_c
     }
 }
 
+// one particle's progress: 4 x (steps done) + phase
+__device__ __forceinline__ int32_t progress(int32_t step, int phase) { return 4 * step + phase; }
+
+// store what phase 1 changed in a step without an event
+__device__ __forceinline__ void store_step(const PushParams &P, int64_t i, const PState<float> &s)
+{
+    const int64_t cap = P.st.cap;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        P.st.F0[k * cap + i] = (double)s.F0[k];
+        P.st.F1[k * cap + i] = (double)s.F1[k];
+    }
+    P.st.vpar[i] = (double)s.vpar0;
+    P.st.s_rem[i] = AccOf<float>::to(s.S);
+    P.st.h_prev[i] = (double)s.hprev;
+    P.st.event[i] = s.event;
+    store_flags(P, i, s.flags);
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(128) split_kernel(const __grid_constant__ Phys<float> ph, const __grid_constant__ SplitParams Q)
 {
@@ -882,10 +908,9 @@ __global__ void __launch_bounds__(128) split_kernel(const __grid_constant__ Phys
     const float dtT = (float)P.dt;
     const StepW<float> w1 = {dtT * 1.5f, dtT * -0.5f, dtT * (float)(2.0 / 3.0), dtT * (float)(5.0 / 12.0),
                              dtT * (float)(-1.0 / 12.0)};
-    const bool on_list = (KIND == SPLIT_R2 || KIND == SPLIT_R3);
     int64_t n = P.st.n;
-    if (on_list) n = *Q.count;
-    if (KIND == SPLIT_INJ_REQ || KIND == SPLIT_INJ_FIX) n = Q.n_new;
+    if (KIND == SPLIT_ROUND && Q.list_in) n = *Q.count_in;
+    if (KIND == SPLIT_INJ_REQ || KIND == SPLIT_INJ_FIX || KIND == SPLIT_INJ_FIN) n = Q.n_new;
     unsigned n_coll = 0, n_reb = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
@@ -894,74 +919,110 @@ __global__ void __launch_bounds__(128) split_kernel(const __grid_constant__ Phys
             put_point(Q.req, k, (float)E.R0[0], (float)E.R0[1], (float)E.R0[2]);
             continue;
         }
-        const int64_t i = on_list ? (int64_t)Q.list[k] : (KIND == SPLIT_INJ_FIX ? Q.slot0 + k : k);
+        int64_t i = k;
+        if (KIND == SPLIT_ROUND && Q.list_in) i = Q.list_in[k];
+        if (KIND == SPLIT_INJ_FIX || KIND == SPLIT_INJ_FIN) i = Q.slot0 + k;
+        int step = 0, phase = 0;
+        if constexpr (KIND == SPLIT_ROUND) {
+            const int32_t pr = Q.prog[i];
+            step = pr >> 2;
+            phase = pr & 3;
+            if (step >= P.n_steps) continue;
+        }
         PConst c;
         PState<float> s;
         load_particle(P, i, c, s);
-        const StepW<float> w = step_weights(w1, dtT, s.hprev);
+        StepW<float> w = step_weights(w1, dtT, s.hprev);
         Sample<float> smp;
         float Fo[4];
         Aux<float> ax;
         float px, py, pz, pu;
         int n_phase = 2;
-        if constexpr (KIND == SPLIT_PRED) {
+        if constexpr (KIND == SPLIT_INIT) {
             phase_point(0, s, w, dtT, px, py, pz, pu);
             put_point(Q.req, i, px, py, pz);
-            continue;
-        } else if constexpr (KIND == SPLIT_CORR) {
-            phase_point(0, s, w, dtT, px, py, pz, pu);
-            load_sample(Q.S, i, Q.g_in_sample, smp);
-            s.flags |= smp.flags;
-            rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
-            phase_consume(0, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, Q.kk, n_coll, n_reb);
-            put_point(Q.req, i, Acc::val(s.Rx), Acc::val(s.Ry), Acc::val(s.Rz));
-            store_RU(P, i, s);
-        } else if constexpr (KIND == SPLIT_POST) {
-            phase_point(1, s, w, dtT, px, py, pz, pu);
-            load_sample(Q.S, i, Q.g_in_sample, smp);
-            s.flags |= smp.flags;
-            rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
-            phase_consume(1, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, Q.kk, n_coll, n_reb);
-            s.hprev = dtT;
-            if (n_phase == 4) {
-                const int32_t slot = atomicAdd(Q.count, 1);
-                Q.list[slot] = (int32_t)i;
-                put_point(Q.reqR, slot, Acc::val(s.Rx), Acc::val(s.Ry), Acc::val(s.Rz));
-            } else {
-                if (!(m_finite(Acc::val(s.Rx)) && m_finite(Acc::val(s.U)) && m_finite(s.F0[0])))
-                    s.flags |= FLAG_NONFINITE;
-                if (Q.tally_now) {
-                    const double t_new = step_time(P.t0, Q.kk, P.dt);
+            Q.prog[i] = progress(0, 0);
+        } else if constexpr (KIND == SPLIT_ROUND) {
+            const long long kk = Q.kbase + step + 1;
+            bool ends = false; // the step is complete
+            if (phase == 0) {
+                phase_point(0, s, w, dtT, px, py, pz, pu);
+                load_sample(Q.S, k, Q.g_in_sample, smp);
+                s.flags |= smp.flags;
+                rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
+                phase_consume(0, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, kk, n_coll, n_reb);
+                px = Acc::val(s.Rx);
+                py = Acc::val(s.Ry);
+                pz = Acc::val(s.Rz);
+                store_RU(P, i, s);
+                phase = 1;
+            } else if (phase == 1) {
+                phase_point(1, s, w, dtT, px, py, pz, pu);
+                load_sample(Q.S, k, Q.g_in_sample, smp);
+                s.flags |= smp.flags;
+                rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
+                phase_consume(1, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, kk, n_coll, n_reb);
+                s.hprev = dtT;
+                if (n_phase == 4) {
+                    px = Acc::val(s.Rx);
+                    py = Acc::val(s.Ry);
+                    pz = Acc::val(s.Rz);
+                    store_particle(P, i, s);
+                    phase = 2;
+                } else {
+                    if (!(m_finite(Acc::val(s.Rx)) && m_finite(Acc::val(s.U)) && m_finite(s.F0[0])))
+                        s.flags |= FLAG_NONFINITE;
+                    if (P.tally_on && (P.step0 + kk) % P.tally.cadence == 0) {
+                        const double t_new = step_time(P.t0, kk, P.dt);
+                        tally_sample<float>(P.tally, P, ph, c.e, Acc::val(s.Rx), Acc::val(s.Ry), Acc::val(s.Rz),
+                                            Acc::val(s.U), s.mub, s.Bm0, t_new - s.t_birth, s.ncoll,
+                                            s.t_birth >= P.tally.t_start && (int)c.e < P.tally.n_ens);
+                    }
+                    store_step(P, i, s);
+                    ends = true;
+                }
+            } else if (phase == 2) {
+                phase_point(2, s, w, dtT, px, py, pz, pu);
+                load_sample(Q.S, k, Q.g_in_sample, smp);
+                s.flags |= smp.flags;
+                rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
+                phase_consume(2, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, kk, n_coll, n_reb);
+                if (P.tally_on && (P.step0 + kk) % P.tally.cadence == 0) {
+                    const double t_new = step_time(P.t0, kk, P.dt);
                     tally_sample<float>(P.tally, P, ph, c.e, Acc::val(s.Rx), Acc::val(s.Ry), Acc::val(s.Rz),
                                         Acc::val(s.U), s.mub, s.Bm0, t_new - s.t_birth, s.ncoll,
                                         s.t_birth >= P.tally.t_start && (int)c.e < P.tally.n_ens);
                 }
+                phase_point(3, s, w, dtT, px, py, pz, pu);
+                store_F(P, i, s, 0);
+                phase = 3;
+            } else {
+                phase_point(3, s, w, dtT, px, py, pz, pu);
+                load_sample(Q.S, k, Q.g_in_sample, smp);
+                s.flags |= smp.flags;
+                rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
+                phase_consume(3, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, kk, n_coll, n_reb);
+                if (!(m_finite(Acc::val(s.Rx)) && m_finite(Acc::val(s.U)) && m_finite(s.F0[0])))
+                    s.flags |= FLAG_NONFINITE;
+                store_F(P, i, s, 1);
+                ends = true;
             }
-            store_particle(P, i, s);
-        } else if constexpr (KIND == SPLIT_R2) {
-            phase_point(2, s, w, dtT, px, py, pz, pu);
-            load_sample(Q.SR, k, Q.g_in_sample, smp);
-            s.flags |= smp.flags;
-            rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
-            phase_consume(2, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, Q.kk, n_coll, n_reb);
-            if (Q.tally_now) {
-                const double t_new = step_time(P.t0, Q.kk, P.dt);
-                tally_sample<float>(P.tally, P, ph, c.e, Acc::val(s.Rx), Acc::val(s.Ry), Acc::val(s.Rz),
-                                    Acc::val(s.U), s.mub, s.Bm0, t_new - s.t_birth, s.ncoll,
-                                    s.t_birth >= P.tally.t_start && (int)c.e < P.tally.n_ens);
+            if (ends) {
+                // the next step's predictor point
+                ++step;
+                phase = 0;
+                w = step_weights(w1, dtT, s.hprev);
+                phase_point(0, s, w, dtT, px, py, pz, pu);
             }
-            phase_point(3, s, w, dtT, px, py, pz, pu);
-            put_point(Q.reqR, k, px, py, pz);
-            store_F(P, i, s, 0);
-        } else if constexpr (KIND == SPLIT_R3) {
-            phase_point(3, s, w, dtT, px, py, pz, pu);
-            load_sample(Q.SR, k, Q.g_in_sample, smp);
-            s.flags |= smp.flags;
-            rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
-            phase_consume(3, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, Q.kk, n_coll, n_reb);
-            if (!(m_finite(Acc::val(s.Rx)) && m_finite(Acc::val(s.U)) && m_finite(s.F0[0])))
-                s.flags |= FLAG_NONFINITE;
-            store_F(P, i, s, 1);
+            Q.prog[i] = progress(step, phase);
+            if (step < P.n_steps) {
+                int64_t slot = k;
+                if (Q.list_out) {
+                    slot = atomicAdd(Q.count_out, 1);
+                    Q.list_out[slot] = (int32_t)i;
+                }
+                put_point(Q.req, slot, px, py, pz);
+            }
         } else if constexpr (KIND == SPLIT_INJ_FIX) {
             // the injection's field-dependent part with this source: mu_B from |B| at the
             // site, F^n there, and the F^{n-1} request at X^n - dt F^n (Sect. 2.2)
@@ -975,18 +1036,26 @@ __global__ void __launch_bounds__(128) split_kernel(const __grid_constant__ Phys
             s.mub = (float)mub;
             mub_lo_set<float>(mub, s.mub);
             rhs(smp, ph, Q.ideal, (float)u, (float)mub, Fo, ax);
-            phase_consume(2, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, Q.kk, n_coll, n_reb);
-            Q.list[k] = (int32_t)i;
+            phase_consume(2, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, 0, n_coll, n_reb);
             phase_point(3, s, w, dtT, px, py, pz, pu);
-            put_point(Q.reqR, k, px, py, pz);
+            put_point(Q.req, k, px, py, pz);
             P.st.u[i] = u;
             P.st.mub[i] = mub;
             P.st.u_inj[i] = u;
             P.st.mub_inj[i] = mub;
             store_F(P, i, s, 0);
+        } else if constexpr (KIND == SPLIT_INJ_FIN) {
+            phase_point(3, s, w, dtT, px, py, pz, pu);
+            load_sample(Q.S, k, Q.g_in_sample, smp);
+            s.flags |= smp.flags;
+            rhs(smp, ph, Q.ideal, pu, s.mub, Fo, ax);
+            phase_consume(3, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, P.t0, 0, n_coll, n_reb);
+            if (!(m_finite(Acc::val(s.Rx)) && m_finite(Acc::val(s.U)) && m_finite(s.F0[0])))
+                s.flags |= FLAG_NONFINITE;
+            store_F(P, i, s, 1);
         }
     }
-    if (KIND == SPLIT_POST) flush_counters(P, n_coll, n_reb);
+    if (KIND == SPLIT_ROUND) flush_counters(P, n_coll, n_reb);
 }
 
 // grid samples in the split-step layout (Sample fields, index-space derivatives with g)
@@ -1111,25 +1180,21 @@ cudaError_t launch_inject(int precision, const GridHost &g, const PhysHost &ph,
     return cudaGetLastError();
 }
 
-cudaError_t launch_split(int kind, const PhysHost &ph, const SplitParams &p, cudaStream_t s)
+cudaError_t launch_split(int kind, const PhysHost &ph, const SplitParams &p, int64_t n, cudaStream_t s)
 {
     const Phys<float> q = make_phys<float>(ph);
-    const int block = 128;
-    int64_t n = p.P.st.n;
-    if (kind == SPLIT_R2 || kind == SPLIT_R3) n = p.P.st.n; // list length known on the device only
-    if (kind == SPLIT_INJ_REQ || kind == SPLIT_INJ_FIX) n = p.n_new;
+    // one warp per block up to an SM's worth of warps each: a round of few particles is latency
+    const int block = n <= 152 * 128 ? 32 : 128;
     int64_t blocks = (n + block - 1) / block;
     if (blocks > 152 * 64) blocks = 152 * 64;
     if (blocks < 1) blocks = 1;
     cudaGetLastError();
     switch (kind) {
-    case SPLIT_PRED: split_kernel<SPLIT_PRED><<<(int)blocks, block, 0, s>>>(q, p); break;
-    case SPLIT_CORR: split_kernel<SPLIT_CORR><<<(int)blocks, block, 0, s>>>(q, p); break;
-    case SPLIT_POST: split_kernel<SPLIT_POST><<<(int)blocks, block, 0, s>>>(q, p); break;
-    case SPLIT_R2: split_kernel<SPLIT_R2><<<(int)blocks, block, 0, s>>>(q, p); break;
-    case SPLIT_R3: split_kernel<SPLIT_R3><<<(int)blocks, block, 0, s>>>(q, p); break;
+    case SPLIT_INIT: split_kernel<SPLIT_INIT><<<(int)blocks, block, 0, s>>>(q, p); break;
+    case SPLIT_ROUND: split_kernel<SPLIT_ROUND><<<(int)blocks, block, 0, s>>>(q, p); break;
     case SPLIT_INJ_REQ: split_kernel<SPLIT_INJ_REQ><<<(int)blocks, block, 0, s>>>(q, p); break;
     case SPLIT_INJ_FIX: split_kernel<SPLIT_INJ_FIX><<<(int)blocks, block, 0, s>>>(q, p); break;
+    case SPLIT_INJ_FIN: split_kernel<SPLIT_INJ_FIN><<<(int)blocks, block, 0, s>>>(q, p); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

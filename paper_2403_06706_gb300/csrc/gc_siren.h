@@ -69,6 +69,4 @@ cudaError_t siren_eval(const SirenNet &net, const SirenIn &in, const SirenOut &o
 cudaError_t train_act_map(CUtensorMap *m, const void *act, int64_t cap);
 cudaError_t train_fwd_bwd(const SirenNet &net, const CUtensorMap &act, const float *x, const float *t, int64_t n,
                           float *G, double *loss, cudaStream_t s);
-// CTAs of the fused evaluation per launch (one per SM)
-int siren_eval_grid(int64_t n);
 } // namespace gcs

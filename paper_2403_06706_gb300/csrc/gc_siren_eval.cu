@@ -52,17 +52,29 @@ using namespace tc;
 
 namespace {
 
-constexpr int kPts = 64;                        // points per tile
 constexpr int kStagesW = 4;                     // weight ring depth
 constexpr uint32_t kChunkBytes = 128u * 128u;   // 128 output rows x 64 bf16
 constexpr uint32_t kW5Bytes = 4u * 16u * 128u;  // W5 padded: 4 boxes of 16 rows x 64 bf16
-constexpr uint32_t kHBytes = 32u * 4u * 1024u;  // 32 K-groups x 4 MN-blocks of 1024 B
 constexpr int kChunksPerTile = 3 * 8;
 constexpr int kComputeWarps = 16;               // arrivals on each h_ready barrier
 constexpr int kThreads = 576;
 constexpr int kMmaWarp = 16, kTmaWarp = 17;
+constexpr int kSmallTiles = 1;  // tiles of 16 points per SM up to which they are taken instead of 64
 constexpr uint32_t kPtsBytes = 16u * 16u * 16u;  // per compute warp: its 16 points as float4
-constexpr size_t kSmemBytes = kHBytes + kStagesW * kChunkBytes + kW5Bytes + kPtsBytes + 1024 + 256;
+
+// A tile of PTS points (64, or 16 for few points): 4 PTS rows, a K-group of 8 features as
+// blocks of 8 features x 64 rows of 1024 B
+template <int PTS>
+struct Tile {
+    static constexpr int kRows = 4 * PTS;
+    static constexpr uint32_t kGroupBytes = kRows / 64 * 1024;
+    static constexpr uint32_t kHBytes = 32 * kGroupBytes;
+    static constexpr int kOutTiles = kRows > 128 ? kRows / 128 : 1; // M-tiles of the output layer
+    static constexpr int kWarpPts = PTS / 4, kWarpRows = kRows / 4;
+    static constexpr int kCols = kWarpRows < 32 ? kWarpRows : 32; // columns per tensor-memory load
+    static constexpr uint32_t kTmemCols = 2 * kRows;
+    static constexpr size_t kSmem = kHBytes + kStagesW * kChunkBytes + kW5Bytes + kPtsBytes + 1024 + 256;
+};
 
 struct EvalParams {
     const float *P;  // master parameters
@@ -148,14 +160,17 @@ __device__ __forceinline__ void store_out(const EvalParams &p, const float (&b5)
     }
 }
 
+template <int PTS>
 __global__ void __launch_bounds__(kThreads, 1)
     siren_eval_kernel(const __grid_constant__ CUtensorMap mwh, const __grid_constant__ CUtensorMap mw5,
                       const __grid_constant__ EvalParams p)
 {
+    using Tl = Tile<PTS>;
+    constexpr uint32_t kGroup = Tl::kGroupBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sH = smem;
-    uint8_t *sW = smem + kHBytes;
+    uint8_t *sW = smem + Tl::kHBytes;
     uint8_t *sW5 = sW + kStagesW * kChunkBytes;  // W5, resident for the whole launch
     float4 *sPts = (float4 *)(sW5 + kW5Bytes);  // [16 compute warps][16 points]
     uint64_t *full = (uint64_t *)(sW5 + kW5Bytes + kPtsBytes);
@@ -176,7 +191,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int64_t nd = *p.in.n_dev;
         n_pts = nd < n_pts ? (nd > 0 ? nd : 0) : n_pts;
     }
-    const int64_t n_tiles = (n_pts + kPts - 1) / kPts;
+    const int64_t n_tiles = (n_pts + PTS - 1) / PTS;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStagesW; ++s) {
@@ -196,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_fence_init();
     }
     if (warp == kMmaWarp) {
-        tmem_alloc(tmem_slot, 512);
+        tmem_alloc(tmem_slot, Tl::kTmemCols);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -244,7 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // high word and a running low word. With descriptors built from addresses for every MMA
         // and the stage found by a division, beside four compute warps on the same scheduler an
         // MMA took 170 cycles to issue against the 128 the tensor cores need for it.
-        constexpr uint32_t id_hid = idesc_bf16_f32(128, 256, 0, 1);
+        constexpr uint32_t id_hid = idesc_bf16_f32(128, Tl::kRows, 0, 1);
         constexpr uint32_t id_out = idesc_bf16_f32(128, 16, 1, 0);
         const bool leader = elect_one();
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
@@ -278,11 +293,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (q == 4 && !wait(&h_ready[1], nh, 13)) { ok = false; break; }
                     if (!wait(&full[st], par, 14)) { ok = false; break; }
                     if (leader) {
-                        const uint32_t a_lo = w_lo + st * (kChunkBytes / 16), b_lo = h_lo + kb * (4 * 8192 / 16);
+                        const uint32_t a_lo = w_lo + st * (kChunkBytes / 16), b_lo = h_lo + kb * (8 * kGroup / 16);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + h * 256, desc_of(desc_hi(1024), a_lo + ks * (32 / 16)),
-                                     desc_of(desc_hi(4096), b_lo + ks * (8192 / 16)), id_hid, (uint32_t)(kb | ks));
+                            mma_bf16(tm + h * Tl::kRows, desc_of(desc_hi(1024), a_lo + ks * (32 / 16)),
+                                     desc_of(desc_hi(kGroup), b_lo + ks * (2 * kGroup / 16)), id_hid,
+                                     (uint32_t)(kb | ks));
                         mma_commit(&empty[st]);
                         // half 0 complete, and with it every MMA of this layer over inputs 0-127
                         if (q == 5) mma_commit(&acc[0]);
@@ -297,18 +313,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ++nh;
             }
             // output layer: rows x W5^T, M-tile 0 into columns 0-15 and M-tile 1 into 16-31
-            // (both in the drained half-0 accumulator), in two K halves: input features
+            // (both in the drained half-0 accumulator; of a 64-row tile's one M-tile the upper
+            // 64 rows read on into the next features, or the ring, and are not used), in two K halves: input features
             // 0-127 as soon as their epilogue is done, 128-255 after the last one
             for (int kh = 0; kh < 2 && ok; ++kh) {
                 if (!wait(&h_ready[kh], nh, 15 + kh)) { ok = false; break; }
                 if (leader) {
                     const uint32_t w5_lo = desc_lo(smem_u32(sW5), 16);
 #pragma unroll
-                    for (int mt = 0; mt < 2; ++mt)
+                    for (int mt = 0; mt < Tl::kOutTiles; ++mt)
 #pragma unroll
                         for (int k8 = 0; k8 < 8; ++k8) {
                             const int k16 = kh * 8 + k8;
-                            mma_bf16(tm + mt * 16, desc_of(desc_hi(4096), h_lo + (mt * 2048 + k16 * 8192) / 16),
+                            mma_bf16(tm + mt * 16, desc_of(desc_hi(kGroup), h_lo + (mt * 2048 + k16 * 2 * kGroup) / 16),
                                      desc_of(desc_hi(1024), w5_lo + ((k16 >> 2) * 2048 + (k16 & 3) * 32) / 16), id_out,
                                      k16 ? 1u : 0u);
                         }
@@ -349,8 +366,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             b5[o] = p.P[siren_oB(5) + o];
         const uint32_t lane_base = tmem + ((uint32_t)(lq * 32) << 16);
         // the feature's 128-byte row in its K-group's first atom, for each half
-        uint8_t *hrow0 = sH + ((lq * 32 + lane) >> 3) * 4096 + (lane & 7) * 128;
-        uint8_t *hrow1 = hrow0 + 16 * 4096;
+        uint8_t *hrow0 = sH + ((lq * 32 + lane) >> 3) * kGroup + (lane & 7) * 128;
+        uint8_t *hrow1 = hrow0 + 16 * kGroup;
         const uint32_t rsw = (uint32_t)(lane & 7);
         uint32_t na0 = 0, na1 = 0, no = 0, noa = 0;
         bool ok = true, first = true;
@@ -359,9 +376,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         // shared-memory slots for the first layer, where every lane reads it by broadcast; the
         // next tile's are fetched while the current one runs
         float px = 0.f, py = 0.f, pz = 0.f;
-        const int pt_off = rg * 16 + (lane & 15);
+        const int pt_off = rg * Tl::kWarpPts + (lane & (Tl::kWarpPts - 1));
+        // this warp's part of the output accumulator (its M-tile rg)
+        const bool outs = rg < Tl::kOutTiles && lq * 32 < Tl::kRows;
         {
-            const int64_t P = (int64_t)blockIdx.x * kPts + pt_off;
+            const int64_t P = (int64_t)blockIdx.x * PTS + pt_off;
             if (P < n_pts) {
                 px = __ldg(p.in.p + 3 * P) * p.in.x_scale;
                 py = __ldg(p.in.p + 3 * P + 1) * p.in.x_scale;
@@ -370,9 +389,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         float4 *wpts = sPts + warp * 16;
         for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-            const int64_t base = t * kPts;
+            const int64_t base = t * PTS;
             __syncwarp();  // every lane done with the previous tile's points
-            if (lane < 16) wpts[lane] = make_float4(px, py, pz, 0.f);
+            if (lane < Tl::kWarpPts) wpts[lane] = make_float4(px, py, pz, 0.f);
             __syncwarp();
             // Layer 1 on the CUDA cores, half 0 then half 1. The previous tile's output layer
             // still runs meanwhile: half 0 overwrites input features 0-127 once the output
@@ -390,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     ++noa;
                 }
 #pragma unroll 2
-                for (int p2 = 0; p2 < 8; ++p2) {
+                for (int p2 = 0; p2 < Tl::kWarpPts / 2; ++p2) {
                     float o[8];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
@@ -409,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         o[4 * e + 2] = wc * w1[h][1];
                         o[4 * e + 3] = wc * w1[h][2];
                     }
-                    store_rows8(hrow, rsw, (uint32_t)(rg * 64 + 8 * p2), o);
+                    store_rows8(hrow, rsw, (uint32_t)(rg * Tl::kWarpRows + 8 * p2), o);
                 }
                 fence_proxy_async_smem();
                 float v[16];
@@ -420,17 +439,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     ++no;
                     tc_fence_after();
-                    if (rg < 2) tmem_ld16(lane_base + rg * 16, v);
+                    if (outs) tmem_ld16(lane_base + rg * 16, v);
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&h_ready[h]);
-                if (h == 0 && !first && rg < 2)
+                if (h == 0 && !first && outs)
                     store_out(p, b5, v, base_prev, rg * 128 + lq * 32 + lane, lane, n_pts);
             }
             if (!ok) break;
             {
-                const int64_t P = (t + gridDim.x) * kPts + pt_off;
+                const int64_t P = (t + gridDim.x) * PTS + pt_off;
                 px = py = pz = 0.f;
                 if (t + gridDim.x < n_tiles && P < n_pts) {
                     px = __ldg(p.in.p + 3 * P) * p.in.x_scale;
@@ -453,19 +472,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float b = bl[L][h];
                     // (half 0: every MMA over inputs 0-127 is complete with its accumulator)
 #pragma unroll 1
-                    for (int c = 0; c < 2; ++c) {
-                        float v[32];
-                        tmem_ld32(lane_base + h * 256 + rg * 64 + c * 32, v);
-                        if (h == 1 && c == 1) {
+                    for (int c = 0; c < Tl::kWarpRows / Tl::kCols; ++c) {
+                        float v[Tl::kCols];
+                        tmem_ld(lane_base + h * Tl::kRows + rg * Tl::kWarpRows + c * Tl::kCols, v);
+                        if (h == 1 && c == Tl::kWarpRows / Tl::kCols - 1) {
                             // the half-1 accumulator is read: the next layer's half-1 MMAs
                             // over inputs 0-127 may run during the rest of this epilogue
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive(h1_drained);
                         }
-                        float o[4][8];
+                        float o[Tl::kCols / 8][8];
 #pragma unroll
-                        for (int pp = 0; pp < 4; ++pp)
+                        for (int pp = 0; pp < Tl::kCols / 8; ++pp)
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 // |z| stays small in the hidden layers: the hardware sine
@@ -479,8 +498,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 o[pp][4 * e + 3] = cs * v[q0 + 3];
                             }
 #pragma unroll
-                        for (int pp = 0; pp < 4; ++pp)
-                            store_rows8(hrow, rsw, (uint32_t)(rg * 64 + c * 32 + 8 * pp), o[pp]);
+                        for (int pp = 0; pp < Tl::kCols / 8; ++pp)
+                            store_rows8(hrow, rsw, (uint32_t)(rg * Tl::kWarpRows + c * Tl::kCols + 8 * pp), o[pp]);
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
@@ -495,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the last tile's output layer
         if (ok && !first && wait_abort(acc_out, no & 1u, abort, p.err, 20)) {
             tc_fence_after();
-            if (rg < 2) {
+            if (outs) {
                 float v[16];
                 tmem_ld16(lane_base + rg * 16, v);
                 store_out(p, b5, v, base_prev, rg * 128 + lq * 32 + lane, lane, n_pts);
@@ -506,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     if (warp == kMmaWarp) {
         tc_fence_after();
-        tmem_dealloc(tmem, 512);
+        tmem_dealloc(tmem, Tl::kTmemCols);
     }
 }
 
@@ -519,7 +538,9 @@ cudaError_t siren_maps(SirenNet &net)
     return e;
 }
 
-int siren_eval_grid(int64_t n)
+namespace {
+
+int sm_count()
 {
     static int n_sm = 0;
     if (!n_sm) {
@@ -528,25 +549,37 @@ int siren_eval_grid(int64_t n)
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (n_sm <= 0) n_sm = 1;
     }
-    const int64_t tiles = (n + kPts - 1) / kPts;
-    return (int)(tiles < n_sm ? tiles : n_sm);
+    return n_sm;
 }
+
+template <int PTS>
+cudaError_t launch_eval(const SirenNet &net, const EvalParams &p, int64_t n, cudaStream_t s)
+{
+    cudaError_t e = cudaFuncSetAttribute(siren_eval_kernel<PTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Tile<PTS>::kSmem);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = (n + PTS - 1) / PTS;
+    const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
+    siren_eval_kernel<PTS><<<grid, kThreads, Tile<PTS>::kSmem, s>>>(net.map_wh, net.map_w5, p);
+    return cudaGetLastError();
+}
+
+} // namespace
 
 cudaError_t siren_eval(const SirenNet &net, const SirenIn &in, const SirenOut &out, cudaStream_t s)
 {
     if (in.n <= 0) return cudaSuccess;
     if (!net.err) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(siren_eval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBytes);
-    if (e != cudaSuccess) return e;
     EvalParams p;
     p.P = net.P;
     p.in = in;
     p.out = out;
     p.omega0 = net.omega0;
     p.err = net.err;
-    siren_eval_kernel<<<siren_eval_grid(in.n), kThreads, kSmemBytes, s>>>(net.map_wh, net.map_w5, p);
-    return cudaGetLastError();
+    // Few points: tiles of 16 spread over the SMs and pass the chain of layers sooner; a count
+    // on the device is expected far below its capacity.
+    if (in.n_dev || in.n <= (int64_t)kSmallTiles * 16 * sm_count()) return launch_eval<16>(net, p, in.n, s);
+    return launch_eval<64>(net, p, in.n, s);
 }
 
 } // namespace gcs
