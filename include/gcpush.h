@@ -167,7 +167,8 @@ typedef struct {
     uint64_t sorts;           /* cell sorts performed */
     double sort_ms;           /* summed device time of the sorts */
     uint64_t field_evals;     /* field samples of the split-step push (points) */
-    double field_ms;          /* summed device time of those sample launches */
+    double field_ms;          /* summed device time of those sample launches (of the whole launch
+                               * where few particles are pushed beside the evaluation) */
 } gc_stats_out;
 
 /* Create a context on opt->device. *out receives the handle. */

@@ -679,7 +679,9 @@ gcp::SplitParams split_params(gc_ctx *c, double dt, double lambda_au)
 // over the list of those that rebirths and collisions held up
 int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool *anomaly)
 {
-    TRY(ensure_split(c));
+    // few particles and the network: whole stretches of steps in one launch
+    const bool one_launch = c->field_source == GC_FIELD_SIREN && gcs::siren_push_fits(c->n);
+    if (!one_launch) TRY(ensure_split(c));
     gcp::SplitParams Q = split_params(c, dt, lambda_au);
     const gcp::PhysHost ph = c->phys();
     cudaStream_t s = c->stream;
@@ -687,6 +689,17 @@ int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool 
     const uint64_t coll0 = c->collisions, reb0 = c->rebirths;
     Q.P.step0 = c->step;
     for (int64_t done = 0; done < n_steps; done += Q.P.n_steps) {
+        if (one_launch) {
+            Q.P.n_steps = (int32_t)std::min<int64_t>(n_steps - done, c->steps_per_launch);
+            Q.P.kbase = done;
+            Timed t;
+            TRY(new_interval(c, 2, nullptr, &t));
+            CUDA_TRY(cudaEventRecord(t.a, s));
+            CUDA_TRY(gcn::neural_push(c->nn, ph, Q.P, c->gh.ideal, s));
+            CUDA_TRY(cudaEventRecord(t.b, s));
+            lc.kernels += 1;
+            continue;
+        }
         Q.P.n_steps = (int32_t)std::min<int64_t>(n_steps - done, 1 << 20);
         Q.kbase = done;
         Q.list_in = Q.count_in = nullptr;

@@ -415,16 +415,37 @@ cudaError_t neural_field(Neural &nn, const float *x, int64_t n, float *field, cu
     return gcs::siren_eval(nn.net, in, o, s);
 }
 
+namespace {
+
+// input and output of an evaluation at positions in m, with the physical field's scaling
+void sample_io(const Neural &nn, const float *R, int64_t cap, const int32_t *n_dev, float *samples, int stride,
+               gcs::SirenIn *in, gcs::SirenOut *o)
+{
+    *in = gcs::SirenIn{R, cap, n_dev, (float)(1.0 / nn.r_max), 1.0f};
+    *o = gcs::SirenOut{};
+    o->field = samples;
+    o->field_stride = stride;
+    o->B_scale = nn.B_scale;
+    o->E_scale = nn.E_scale;
+}
+
+} // namespace
+
 cudaError_t neural_field_at(Neural &nn, const float *R, int64_t cap, const int32_t *n_dev, float *samples,
                             int stride, cudaStream_t s)
 {
-    gcs::SirenIn in{R, cap, n_dev, (float)(1.0 / nn.r_max), 1.0f};
-    gcs::SirenOut o{};
-    o.field = samples;
-    o.field_stride = stride;
-    o.B_scale = nn.B_scale;
-    o.E_scale = nn.E_scale;
+    gcs::SirenIn in;
+    gcs::SirenOut o;
+    sample_io(nn, R, cap, n_dev, samples, stride, &in, &o);
     return gcs::siren_eval(nn.net, in, o, s);
+}
+
+cudaError_t neural_push(Neural &nn, const gcp::PhysHost &phys, const gcp::PushParams &push, int ideal, cudaStream_t s)
+{
+    gcs::SirenIn in;
+    gcs::SirenOut o;
+    sample_io(nn, nullptr, push.st.n, nullptr, nullptr, gcp::kSampleStride, &in, &o);
+    return gcs::siren_push(nn.net, in, o, phys, push, ideal, s);
 }
 
 cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, int64_t n, float *out, cudaStream_t s)

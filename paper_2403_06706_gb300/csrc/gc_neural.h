@@ -54,6 +54,8 @@ cudaError_t neural_field(Neural &nn, const float *x, int64_t n, float *field, cu
 // when null), samples with `stride` floats per point
 cudaError_t neural_field_at(Neural &nn, const float *R, int64_t cap, const int32_t *n_dev, float *samples,
                             int stride, cudaStream_t s);
+// the push of few particles with the network's field in one launch (see gcs::siren_push)
+cudaError_t neural_push(Neural &nn, const gcp::PhysHost &phys, const gcp::PushParams &push, int ideal, cudaStream_t s);
 // scaled 8-channel targets of the grid interpolant at x (n x 3, scaled by r_max)
 cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, int64_t n, float *t,
                            cudaStream_t s);

@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "gc_internal.h"
+
 namespace gcs {
 // C = A B^T (+= with atomic != 0) for bf16 A (M x K) and B (N x K), each stored K-major
 // (row-major M x K / N x K) or, with a_mn / b_mn set, MN-major (row-major K x M / K x N);
@@ -63,6 +65,12 @@ struct SirenIn {
 cudaError_t siren_maps(SirenNet &net);
 // evaluate the network (and its Jacobian) at the input points (device)
 cudaError_t siren_eval(const SirenNet &net, const SirenIn &in, const SirenOut &out, cudaStream_t s);
+// The push of few particles (siren_push_fits) with this field in one launch: push.n_steps
+// steps from push.kbase steps into the call (push.t0, push.step0: the call's start); in and
+// out give the scaling and the sample layout, their pointers are not used.
+bool siren_push_fits(int64_t n);
+cudaError_t siren_push(const SirenNet &net, const SirenIn &in, const SirenOut &out, const gcp::PhysHost &phys,
+                       const gcp::PushParams &push, int ideal, cudaStream_t s);
 // Training (gc_train.cu): adds the gradient of the mean squared error of n samples (n a
 // multiple of 64) to G and the sum of squared residuals to loss. act: tensor map, made by
 // train_act_map, of a BF16 work buffer of 6 x 256 rows of `cap` >= n samples (h1..h3, dz2..dz4).
