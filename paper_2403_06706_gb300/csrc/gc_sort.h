@@ -34,7 +34,7 @@ cudaError_t sort_preload();
 cudaError_t alloc_state(StateDev &s, int64_t cap);
 void free_state_arrays(StateDev &s);
 // kernels launched by one sort_by_cell / unpermute_to_alt call
-constexpr int kSortKernels = 3;
+constexpr int kSortKernels = 4;
 constexpr int kUnpermuteKernels = 1;
 
 } // namespace gcp
