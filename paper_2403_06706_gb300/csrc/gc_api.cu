@@ -677,7 +677,7 @@ gcp::SplitParams split_params(gc_ctx *c, double dt, double lambda_au)
 
 // n_steps steps of the split-step push: two rounds per step over all particles, then rounds
 // over the list of those that rebirths and collisions held up
-int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool *anomaly)
+int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool *anomaly, int *tc_error)
 {
     // few particles and the network: whole stretches of steps in one launch
     const bool one_launch = c->field_source == GC_FIELD_SIREN && gcs::siren_push_fits(c->n);
@@ -735,7 +735,9 @@ int split_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au, bool 
         }
     }
     add_counts(c, lc);
+    if (c->field_source == GC_FIELD_SIREN) CUDA_TRY(gcn::neural_status_copy(c->nn, s));
     TRY(collect_status(c, anomaly));
+    if (c->field_source == GC_FIELD_SIREN) *tc_error = gcn::neural_error(c->nn, s);
     c->field_evals += (uint64_t)(2 * c->n * n_steps) + 2 * ((c->collisions - coll0) + (c->rebirths - reb0));
     return GC_OK;
 }
@@ -1102,8 +1104,9 @@ int gc_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au)
         return GC_OK;
     }
     bool anomaly = false;
+    int tc_error = 0;
     if (c->field_source != GC_FIELD_GRID) {
-        TRY(split_advance(c, dt, n_steps, lambda_au, &anomaly));
+        TRY(split_advance(c, dt, n_steps, lambda_au, &anomaly, &tc_error));
     } else if (c->use_graph) {
         TRY(advance_graph(c, dt, n_steps, lambda_au, &anomaly));
     } else {
@@ -1115,6 +1118,8 @@ int gc_advance(gc_ctx *c, double dt, int64_t n_steps, double lambda_au)
     c->t += (double)n_steps * dt;
     c->step += n_steps;
     c->particle_steps += (uint64_t)c->n * (uint64_t)n_steps;
+    if (tc_error)
+        return fail(GC_ERR_DEVICE_ANOMALY, "gc_advance: a tensor-core pipeline wait ran out (code %d)", tc_error);
     if (anomaly)
         return fail(GC_ERR_DEVICE_ANOMALY, "gc_advance: particles flagged (0x%x)", c->flags_or);
     return GC_OK;
@@ -1421,16 +1426,22 @@ int gc_particles_set(gc_ctx *c, const gc_particle_soa *in)
     for (const uint32_t *p : usrc)
         if (!p && in->n) return fail(GC_ERR_INVALID, "gc_particles_set: every array is required");
     const int64_t n = in->n;
-    bool ascending = true;
-    uint32_t lo = 0xFFFFFFFFu, hi = 0;
+    // whole-array reductions without an early exit, which the compiler vectorises (particle by
+    // particle this took 2.5 ms of host time for 3 x 10^6)
+    uint32_t lo = 0xFFFFFFFFu, hi = 0, ens_hi = 0, steps_back = 0;
     for (int64_t k = 0; k < n; ++k) {
-        if (in->ens[k] >= c->ens.size())
-            return fail(GC_ERR_INVALID, "gc_particles_set: particle %lld has unknown ensemble %u",
-                        (long long)k, in->ens[k]);
-        if (k && in->id[k] <= in->id[k - 1]) ascending = false;
+        ens_hi = std::max(ens_hi, in->ens[k]);
         lo = std::min(lo, in->id[k]);
         hi = std::max(hi, in->id[k]);
     }
+    for (int64_t k = 1; k < n; ++k)
+        steps_back |= (uint32_t)(in->id[k] <= in->id[k - 1]);
+    const bool ascending = steps_back == 0;
+    if (n && ens_hi >= c->ens.size())
+        for (int64_t k = 0; k < n; ++k)
+            if (in->ens[k] >= c->ens.size())
+                return fail(GC_ERR_INVALID, "gc_particles_set: particle %lld has unknown ensemble %u",
+                            (long long)k, in->ens[k]);
     bool dense = (n == 0) || ((int64_t)hi - (int64_t)lo + 1 == n);
     if (dense && !ascending) {
         std::vector<char> seen(n, 0);
@@ -1551,9 +1562,9 @@ int gc_siren_get(gc_ctx *c, float *params_host)
 
 static int nn_check_tc(gc_ctx *c, const char *who)
 {
+    CUDA_TRY(gcn::neural_status_copy(c->nn, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
-    int te = gcs::read_error(c->stream);
-    if (!te) te = gcn::neural_read_error(c->nn, c->stream);
+    const int te = gcn::neural_error(c->nn, c->stream);
     if (te) return fail(GC_ERR_DEVICE_ANOMALY, "%s: a tensor-core pipeline wait ran out (code %d)", who, te);
     return GC_OK;
 }
@@ -1594,10 +1605,9 @@ int gc_siren_loss_grad(gc_ctx *c, const float *x_dev, const float *t_dev, int64_
     if (!x_dev || !t_dev || n <= 0 || n % 128 != 0 || n > ((int64_t)1 << 30))
         return fail(GC_ERR_INVALID, "gc_siren_loss_grad: need device x and t and n a positive multiple of 128");
     TRY(set_device(c));
-    double loss = 0.0;
-    CUDA_TRY(gcn::neural_loss_grad(c->nn, x_dev, t_dev, n, grad_dev, &loss, c->stream));
+    CUDA_TRY(gcn::neural_loss_grad(c->nn, x_dev, t_dev, n, grad_dev, c->stream));
     TRY(nn_check_tc(c, "gc_siren_loss_grad"));
-    if (loss_out) *loss_out = loss;
+    if (loss_out) *loss_out = c->nn.h_status->loss / (double)(n * 8);
     return GC_OK;
 }
 

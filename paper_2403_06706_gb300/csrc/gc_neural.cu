@@ -334,16 +334,17 @@ cudaError_t ensure_work(Neural &nn, int64_t rows)
 cudaError_t fwd_bwd(Neural &nn, const float *x, const float *t, int64_t n, float *grad, cudaStream_t s)
 {
     const cudaError_t e = ensure_work(nn, n);
-    return e != cudaSuccess ? e : gcs::train_fwd_bwd(nn.net, nn.map_act, x, t, n, grad, nn.d_loss, s);
+    return e != cudaSuccess ? e : gcs::train_fwd_bwd(nn.net, nn.map_act, x, t, n, grad, &nn.d_status->loss, s);
 }
 
 } // namespace
 
 cudaError_t neural_free(Neural &nn)
 {
-    void *ptrs[] = {nn.P, nn.G, nn.Mo, nn.Vo, nn.Wh, nn.W5p, nn.act, nn.d_loss, nn.d_err, nn.Xs, nn.Ts};
+    void *ptrs[] = {nn.P, nn.G, nn.Mo, nn.Vo, nn.Wh, nn.W5p, nn.act, nn.d_status, nn.Xs, nn.Ts};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (nn.h_status) cudaFreeHost(nn.h_status);
     nn = Neural{};
     return cudaSuccess;
 }
@@ -360,9 +361,9 @@ cudaError_t neural_set(Neural &nn, const float *params, bool on_device, double o
         if (e == cudaSuccess) e = dev_alloc(&nn.Vo, pb);
         if (e == cudaSuccess) e = dev_alloc(&nn.Wh, (size_t)3 * 65536 * sizeof(__nv_bfloat16));
         if (e == cudaSuccess) e = dev_alloc(&nn.W5p, (size_t)16 * 256 * sizeof(__nv_bfloat16));
-        if (e == cudaSuccess) e = dev_alloc(&nn.d_loss, sizeof(double));
-        if (e == cudaSuccess) e = dev_alloc(&nn.d_err, sizeof(int));
-        if (e == cudaSuccess) e = cudaMemsetAsync(nn.d_err, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = dev_alloc(&nn.d_status, sizeof(NeuralStatus));
+        if (e == cudaSuccess) e = cudaMallocHost((void **)&nn.h_status, sizeof(NeuralStatus));
+        if (e == cudaSuccess) e = cudaMemsetAsync(nn.d_status, 0, sizeof(NeuralStatus), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(nn.W5p, 0, (size_t)16 * 256 * sizeof(__nv_bfloat16), s);
         if (e != cudaSuccess) {
             neural_free(nn);
@@ -371,7 +372,7 @@ cudaError_t neural_set(Neural &nn, const float *params, bool on_device, double o
         nn.net.P = nn.P;
         nn.net.Wh = nn.Wh;
         nn.net.W5p = nn.W5p;
-        nn.net.err = nn.d_err;
+        nn.net.err = &nn.d_status->err;
         e = gcs::siren_maps(nn.net);
         if (e != cudaSuccess) {
             neural_free(nn);
@@ -465,30 +466,23 @@ cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, i
     return cudaGetLastError();
 }
 
-cudaError_t neural_loss_grad(Neural &nn, const float *x, const float *t, int64_t n, float *grad, double *loss,
-                             cudaStream_t s)
+cudaError_t neural_loss_grad(Neural &nn, const float *x, const float *t, int64_t n, float *grad, cudaStream_t s)
 {
     float *g = grad ? grad : nn.G;
     cudaError_t e = cudaMemsetAsync(g, 0, (size_t)kSirenNParams * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(nn.d_loss, 0, sizeof(double), s);
-    if (e == cudaSuccess) e = fwd_bwd(nn, x, t, n, g, s);
-    if (e != cudaSuccess) return e;
-    if (loss) {
-        double v = 0.0;
-        e = cudaMemcpyAsync(&v, nn.d_loss, sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        *loss = v / (double)(n * 8);
-    }
-    return e;
+    if (e == cudaSuccess) e = cudaMemsetAsync(&nn.d_status->loss, 0, sizeof(double), s);
+    return e == cudaSuccess ? fwd_bwd(nn, x, t, n, g, s) : e;
 }
 
-int neural_read_error(Neural &nn, cudaStream_t s)
+cudaError_t neural_status_copy(Neural &nn, cudaStream_t s)
 {
-    int v = 0;
-    if (!nn.d_err) return 0;
-    if (cudaMemcpyAsync(&v, nn.d_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return -1;
-    if (v && cudaMemsetAsync(nn.d_err, 0, sizeof(int), s) != cudaSuccess) return -1;
+    return cudaMemcpyAsync(nn.h_status, nn.d_status, sizeof(NeuralStatus), cudaMemcpyDeviceToHost, s);
+}
+
+int neural_error(Neural &nn, cudaStream_t s)
+{
+    const int v = nn.h_status->err;
+    if (v && cudaMemsetAsync(&nn.d_status->err, 0, sizeof(int), s) != cudaSuccess) return -1;
     return v;
 }
 
@@ -525,17 +519,16 @@ cudaError_t neural_fit(Neural &nn, const GridRef &g, const float *samples, bool 
     const int64_t nb = n_samples / batch;
     e = cudaMemsetAsync(nn.G, 0, (size_t)kSirenNParams * sizeof(float), s);
     for (int ep = 0; ep < n_epochs; ++ep) {
-        if (e == cudaSuccess) e = cudaMemsetAsync(nn.d_loss, 0, sizeof(double), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(&nn.d_status->loss, 0, sizeof(double), s);
         for (int64_t b = 0; b < nb && e == cudaSuccess; ++b) {
             e = fwd_bwd(nn, nn.Xs + b * batch * 3, nn.Ts + b * batch * 8, batch, nn.G, s);
             if (e == cudaSuccess) e = neural_adam(nn, lr, beta1, beta2, eps, s);
         }
         if (e != cudaSuccess) return e;
-        double v = 0.0;
-        e = cudaMemcpyAsync(&v, nn.d_loss, sizeof(double), cudaMemcpyDeviceToHost, s);
+        e = neural_status_copy(nn, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return e;
-        if (loss_out) loss_out[ep] = (float)(v / (double)(nb * batch * 8));
+        if (loss_out) loss_out[ep] = (float)(nn.h_status->loss / (double)(nb * batch * 8));
     }
     return cudaSuccess;
 }

@@ -19,6 +19,12 @@ struct GridRef {
     double r_min, dr;
 };
 
+// What the host reads back after evaluations and training, in one copy.
+struct NeuralStatus {
+    double loss;  // sum of squared residuals
+    int err, pad; // error word of the evaluation and training kernels (0: none)
+};
+
 struct Neural {
     bool ready = false;
     float *P = nullptr;   // FP32 master parameters
@@ -35,8 +41,7 @@ struct Neural {
     int64_t wcap = 0;
     __nv_bfloat16 *act = nullptr;
     CUtensorMap map_act{};
-    double *d_loss = nullptr;    // [1]
-    int *d_err = nullptr;        // error word of the fused evaluation and training
+    NeuralStatus *d_status = nullptr, *h_status = nullptr; // device words and their pinned mirror
 
     // fit: samples and targets
     float *Xs = nullptr, *Ts = nullptr;
@@ -59,11 +64,13 @@ cudaError_t neural_push(Neural &nn, const gcp::PhysHost &phys, const gcp::PushPa
 // scaled 8-channel targets of the grid interpolant at x (n x 3, scaled by r_max)
 cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, int64_t n, float *t,
                            cudaStream_t s);
-// mean-squared error over n samples (n a multiple of 128) and its gradient into grad (or nn.G)
-cudaError_t neural_loss_grad(Neural &nn, const float *x, const float *t, int64_t n, float *grad, double *loss,
-                             cudaStream_t s);
-// error word of the fused evaluation (0 = none); reading clears it (synchronises s)
-int neural_read_error(Neural &nn, cudaStream_t s);
+// mean-squared error over n samples (n a multiple of 128) into the status' loss, as the sum of
+// squared residuals, and its gradient into grad (or nn.G)
+cudaError_t neural_loss_grad(Neural &nn, const float *x, const float *t, int64_t n, float *grad, cudaStream_t s);
+// enqueue the copy of the status words to nn.h_status (valid once s is synchronised)
+cudaError_t neural_status_copy(Neural &nn, cudaStream_t s);
+// error word of the copy; an error is cleared on the device
+int neural_error(Neural &nn, cudaStream_t s);
 // one Adam step on nn.G
 cudaError_t neural_adam(Neural &nn, double lr, double beta1, double beta2, double eps, cudaStream_t s);
 // training: targets from the grid, then n_epochs passes of batches (the last partial batch
