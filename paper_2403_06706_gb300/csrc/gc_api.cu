@@ -184,7 +184,7 @@ struct gc_ctx {
     // launch shape
     int block = 0;           // 0: see push_block
     int grid_waves = 1;      // resident waves of blocks (0: one thread per particle)
-    int blocks_per_sm[5] = {0, 0, 0, 0, 0}; // occupancy per block size / 32, cached
+    int blocks_per_sm[17] = {}; // occupancy per block size / 32, cached
     int steps_per_launch = 2000;
     int sort_every = 0;
     int64_t steps_since_sort = 0;
@@ -377,15 +377,12 @@ int blocks_per_sm(gc_ctx *c, int block)
     return nb;
 }
 
-// Threads per block of the push: what gc_set_launch or the autotuner chose, else 32 while one
-// resident wave holds all particles (warps then spread evenly over the SMs: FP32 of 40 000
-// particles 1.78e10 -> 1.88e10 particle-steps/s, FP64 of 4096 / 30 000 1.43e8 -> 1.54e8 /
-// 5.4e8 -> 6.1e8) and 128 beyond (neighbouring groups of particles, which share cells, on one
-// SM: 64 ensembles at as many sites run 23 % slower with 32).
+// Threads per block of the push: what gc_set_launch or the autotuner chose, else one block per
+// SM (FP32 of 934 000 particles 2.88e10 particle-steps/s with blocks of 128, 2.91e10 of 256,
+// 2.99e10 of 512; two-fluid field and wind 2.14e10, 2.17e10, 2.25e10).
 int push_block(gc_ctx *c)
 {
-    if (c->block) return c->block;
-    return c->n <= (int64_t)c->sm_count * blocks_per_sm(c, 128) * 128 ? 32 : 128;
+    return c->block ? c->block : gcp::push_threads(c->opt.precision, c->gh.nodes1 != nullptr);
 }
 
 int push_grid(gc_ctx *c, int block)
@@ -394,7 +391,10 @@ int push_grid(gc_ctx *c, int block)
     const int64_t want = (c->n + block - 1) / block;
     if (c->grid_waves <= 0)
         return (int)std::min<int64_t>(want, 0x7FFFFFFF);
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)c->grid_waves * c->sm_count * nb));
+    const int64_t wave = (int64_t)c->grid_waves * c->sm_count * nb;
+    // one wave is spread over all SMs (push_spread), down to 32 particles per block
+    const bool spread = c->grid_waves == 1 && block % 128 == 0;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(spread ? (c->n + 31) / 32 : want, wave));
 }
 
 // Enqueue the launches of one advance on stream s: cell sorts on schedule and push
@@ -424,6 +424,8 @@ int enqueue_advance(gc_ctx *c, cudaStream_t s, double dt, int64_t n_steps, doubl
     P.gflags = c->d_flags;
     P.counters = c->d_counters;
     P.clock = clock_dev;
+    P.spread_from = INT64_MAX;
+    if (c->grid_waves == 1) gcp::push_spread(P, block, grid);
     const gcp::PhysHost ph = c->phys();
 
     int64_t done = 0;

@@ -42,6 +42,8 @@ struct PushParams {
     double dt, t0;       // t_new = t0 + (kbase + k + 1) dt for local step k
     int64_t step0;       // global step index of local step 0
     int64_t kbase;
+    int64_t spread_from; // first particle not in a full round of the grid (see push_kernel);
+                         // INT64_MAX: whole blocks throughout
     int32_t n_steps;
     int32_t collision_form, no_scatter, no_rebirth;
     double lambda_override; // m, > 0 overrides the ensembles
@@ -113,6 +115,10 @@ cudaError_t launch_push(int precision, const GridHost &g, const PhysHost &ph, co
                         int block, int grid, cudaStream_t s);
 cudaError_t launch_inject(int precision, const GridHost &g, const PhysHost &ph,
                           const InjectParams &p, cudaStream_t s);
+// set the spread of the last round for a grid of one resident wave (p.st.n is set)
+void push_spread(PushParams &p, int block, int grid);
+// most threads per block of the push, as many as an SM holds of it
+int push_threads(int precision, bool time_dependent);
 int push_max_blocks_per_sm(int precision, int block, bool time_dependent = false, bool potential = false);
 // one split-step kernel (FP32 path) over n particles or list entries (at most)
 cudaError_t launch_split(int kind, const PhysHost &ph, const SplitParams &p, int64_t n, cudaStream_t s);

@@ -245,13 +245,14 @@ extern "C" int gc_advance_noalloc(const gc_options *opt, const gc_grid_desc *g, 
     P.gflags = d_flags;
     P.counters = d_counters;
 
-    const int block = 128;
+    const int block = gcp::push_threads(opt->precision, false); // one block per SM, as gc_advance
     int nb = gcp::push_max_blocks_per_sm(opt->precision, block, false, g->ideal == 2);
     cudaGetLastError(); // the occupancy query's status is not this call's
     if (nb < 1) nb = 1;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, opt->device);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((sd->n + block - 1) / block, (int64_t)sms * nb));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((sd->n + 31) / 32, (int64_t)sms * nb));
+    gcp::push_spread(P, block, grid);
     int64_t done = 0;
     while (sd->n > 0 && done < n_steps) {
         const int64_t chunk = std::min<int64_t>(n_steps - done, 2000);

@@ -41,36 +41,20 @@ __device__ __noinline__ Restart<T> restart_history(const GridMeta<T> &gm, const 
 }
 
 // ----------------------------------------------------------------------------------------
-// Resident CTAs of 128 threads per SM the FP32 push is compiled for (register budget:
-// 65536 / (128 x blocks) per thread); the time-dependent variant carries more state.
-#ifndef GC_PUSH_F32_MIN_BLOCKS
-#define GC_PUSH_F32_MIN_BLOCKS 4
-#endif
-constexpr int kMinBlocksF32 = GC_PUSH_F32_MIN_BLOCKS;
-// Time-dependent fields: 3 (4 spilled 172 bytes and measured 6 % slower). Potential channel:
-// 4 like the steady kernel (3 measured 5 % slower).
-#ifndef GC_PUSH_F32_TD_MIN_BLOCKS
-#define GC_PUSH_F32_TD_MIN_BLOCKS 3
-#endif
-constexpr int kMinBlocksF32TD = GC_PUSH_F32_TD_MIN_BLOCKS;
-#ifndef GC_PUSH_F32_POT_MIN_BLOCKS
-#define GC_PUSH_F32_POT_MIN_BLOCKS GC_PUSH_F32_MIN_BLOCKS
-#endif
-constexpr int kMinBlocksF32Pot = GC_PUSH_F32_POT_MIN_BLOCKS;
-// FP64: 2 (3 and 4 spill and measured 0.4 % and 1.7 % slower: the FP64 pipe, not
-// latency, bounds that kernel)
-#ifndef GC_PUSH_F64_MIN_BLOCKS
-#define GC_PUSH_F64_MIN_BLOCKS 2
-#endif
-constexpr int kMinBlocksF64 = GC_PUSH_F64_MIN_BLOCKS;
+// Threads of the push resident per SM, which its register budget (65536 / threads) allows and
+// one block may hold. FP32: 512 (640 at 96 registers spill 48 bytes and measured 1.5 % slower,
+// also with the rarely used state in shared memory; 384 for the potential channel 5 % slower);
+// time-dependent fields 384 (512 spilled 172 bytes and measured 6 % slower). FP64: 256 (384
+// and 512 spill and measured 0.4 % and 1.7 % slower: the FP64 pipe, not latency, bounds it).
+template <typename T, bool TD>
+constexpr int kPushThreads = sizeof(T) == 4 ? (TD ? 384 : 512) : 256;
 
 // Fused push: one thread owns a particle for all the steps of a launch and evaluates the
 // grid field inline.
 template <typename T, bool TD, int POT>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (TD ? kMinBlocksF32TD : (POT == POT_ON ? kMinBlocksF32Pot : kMinBlocksF32)) : kMinBlocksF64) push_kernel(const __grid_constant__ GridMeta<T> gm, const __grid_constant__ Phys<T> ph,
+__global__ void __launch_bounds__((kPushThreads<T, TD>), 1) push_kernel(const __grid_constant__ GridMeta<T> gm, const __grid_constant__ Phys<T> ph,
                                                    const __grid_constant__ PushParams P)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     unsigned n_coll = 0, n_reb = 0;
     const T dtT = (T)P.dt;
     double t0 = P.t0;
@@ -89,7 +73,19 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (TD ? kMinBlocksF32TD : 
     // loop over the phases (unrolled, they spill)
     constexpr bool kUnrollPhases = !TD;
 
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P.st.n; i += stride) {
+    // Particles of the full rounds in blocks of neighbours (which share cells); those left from
+    // P.spread_from on, all of a small population, in groups of kSpread, one per block in turn:
+    // a partial round then has its warps on all SMs. (With whole blocks 200 000 particles, 2.57
+    // rounds of one block of 512 per SM, ran 11 % slower than with blocks of 128; groups of 32
+    // instead of 128 3 % slower, but 8 % faster in FP64 where an SM gets fewer than four warps.)
+    constexpr unsigned kSpread = sizeof(T) == 8 ? 32 : 128;
+    int64_t next = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (;;) {
+        if (next >= P.spread_from)
+            next = P.spread_from + ((int64_t)(threadIdx.x / kSpread) * gridDim.x + blockIdx.x) * kSpread + threadIdx.x % kSpread;
+        if (next >= P.st.n)
+            break;
+        const uint32_t i = (uint32_t)next; // ids, and so slots, have 32 bits
         PConst c;
         PState<T> s;
         load_particle(P, i, c, s);
@@ -154,6 +150,9 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (TD ? kMinBlocksF32TD : 
         if (!(m_finite(AccOf<T>::val(s.Rx)) && m_finite(AccOf<T>::val(s.U)) && m_finite(s.F0[0])))
             s.flags |= FLAG_NONFINITE;
         store_particle(P, i, s);
+        if (i >= P.spread_from)
+            break;
+        next = (int64_t)i + (int64_t)gridDim.x * blockDim.x;
     }
     // counters: one atomic per warp
     const unsigned mask = __activemask();
@@ -460,10 +459,22 @@ InjectFn<T> inject_fn(bool td, bool pot)
     return pot ? inject_kernel<T, false, POT_ON> : inject_kernel<T, false, POT_NONE>;
 }
 
+int push_threads(int precision, bool time_dependent)
+{
+    if (precision == 0) return time_dependent ? kPushThreads<double, true> : kPushThreads<double, false>;
+    return time_dependent ? kPushThreads<float, true> : kPushThreads<float, false>;
+}
+
+void push_spread(PushParams &p, int block, int grid)
+{
+    const int64_t round = (int64_t)grid * block;
+    p.spread_from = block % 128 == 0 ? p.st.n / round * round : INT64_MAX;
+}
+
 cudaError_t launch_push(int precision, const GridHost &g, const PhysHost &ph, const PushParams &p,
                         int block, int grid, cudaStream_t s)
 {
-    if (block < 1 || block > kMaxPushBlock)
+    if (block < 1 || block > push_threads(precision, g.nodes1 != nullptr))
         return cudaErrorInvalidConfiguration;
     cudaGetLastError(); // report this launch only
     const bool td = g.nodes1 != nullptr, pot = g.ideal == 2, ideal = g.ideal == 1;

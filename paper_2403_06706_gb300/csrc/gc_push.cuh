@@ -193,7 +193,7 @@ __device__ __noinline__ void tally_sample(const TallyDev &T_, const PushParams &
 // and store touch, kept in a per-thread shared-memory slot instead of a register the step
 // loop would carry. Blocks of the push kernels have at most kMaxPushBlock threads; the kernel
 // that pushes beside the network's evaluation does so in one warp.
-constexpr int kMaxPushBlock = 128;
+constexpr int kMaxPushBlock = 512; // a power of two
 __shared__ float s_mub_lo[kMaxPushBlock];
 
 template <typename T>
