@@ -105,6 +105,17 @@ __device__ __forceinline__ float m_div(float a, float b) { return __fdividef(a, 
 __device__ __forceinline__ double m_div(double a, double b) { return a / b; }
 __device__ __forceinline__ bool m_finite(float a) { return isfinite(a); }
 __device__ __forceinline__ bool m_finite(double a) { return isfinite(a); }
+// Sums of products with their rounding written out: which product of a sum is rounded by
+// itself is otherwise the compiler's choice, which moves with changes of the code around it
+// (the FP32 push then differs by 1e-7 between two builds of the same formulas).
+__device__ __forceinline__ float m_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double m_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float m_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double m_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float m_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double m_add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float m_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double m_sub(double a, double b) { return __dsub_rn(a, b); }
 template <typename T> __device__ __forceinline__ T two_pi();
 template <> __device__ __forceinline__ float two_pi<float>() { return 6.28318530717958647692f; }
 template <> __device__ __forceinline__ double two_pi<double>() { return 6.28318530717958647692; }
@@ -167,6 +178,10 @@ __device__ __forceinline__ void polar_angles(double x, double y, double z, doubl
     theta = refine_angle(z, rho, inv_r, m_atan2((float)rho, (float)z));
     phi = refine_angle(x, y, inv_rho, m_atan2((float)y, (float)x));
 }
+
+// The evaluations of a step associate the two radii's sums differently (as the FP32 push's
+// results have had them): EV_OTHER stands for injections, restarts and field samples.
+enum : int { EV_OTHER = 0, EV_PREDICTOR, EV_CORRECTOR };
 
 // ----------------------------------------------------------------------------------------
 // Grid description in the precision of the push.
@@ -371,24 +386,24 @@ __device__ __forceinline__ void interp_nodes(const T *__restrict__ nodes, uint32
 // the interpolant (Sect. 2.2). Node-centred grid, poles included in theta, periodic in phi.
 // Positions more than one radial cell outside the grid are flagged; beyond the edge nodes
 // the interpolant is extended as a constant.
-template <typename T, int POT = POT_RUNTIME>
+template <typename T, int POT = POT_RUNTIME, int EV = EV_OTHER>
 __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sample<T> &s,
                                        Sample<T> *s1 = nullptr)
 {
     uint32_t flags = 0;
-    T rho2 = x * x + y * y;
+    T rho2 = EV == EV_OTHER ? m_fma(x, x, m_mul(y, y)) : m_fma(y, y, m_mul(x, x));
     if (!(rho2 > T(1e-30))) {
         flags |= FLAG_AXIS;
         rho2 = T(1e-30);
     }
-    const T r2 = rho2 + z * z;
+    const T r2 = EV == EV_CORRECTOR && POT != POT_ON ? m_add(rho2, m_mul(z, z)) : m_fma(z, z, rho2);
     const T inv_rho = m_rsqrt(rho2), inv_r = m_rsqrt(r2);
     const T rho = rho2 * inv_rho, r = r2 * inv_r;
     T theta, phi;
     polar_angles(x, y, z, rho, inv_rho, inv_r, theta, phi);
     if (phi < T(0))
         phi += two_pi<T>();
-    T xr = (r - gm.r_min) * gm.inv_dr;
+    T xr = m_mul(m_fma(r2, inv_r, -gm.r_min), gm.inv_dr);
     T xt = theta * gm.inv_dth;
     T xp = phi * gm.inv_dph;
     if (!(m_finite(xr) && m_finite(xt) && m_finite(xp))) {
@@ -400,17 +415,17 @@ __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sam
 
     const T flr = m_floor(xr);
     int i = (int)flr;
-    T fr = xr - flr;
+    T fr = m_sub(xr, flr);
     if (i < 0) { i = 0; fr = T(0); }
     else if (i > gm.n_r - 2) { i = gm.n_r - 2; fr = T(1); }
     const T flt = m_floor(xt);
     int j = (int)flt;
-    T ft = xt - flt;
+    T ft = m_sub(xt, flt);
     if (j < 0) { j = 0; ft = T(0); }
     else if (j > gm.n_th - 2) { j = gm.n_th - 2; ft = T(1); }
     const T flp = m_floor(xp);
     int k = (int)flp;
-    const T fp = xp - flp;
+    const T fp = m_sub(xp, flp);
     if (k >= gm.n_ph) k -= gm.n_ph;
     if (k < 0) k += gm.n_ph;
     const int k1 = (k + 1 == gm.n_ph) ? 0 : k + 1;
@@ -440,11 +455,11 @@ __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sam
 // quantity blended linearly at t_rel seconds after the first snapshot (held constant
 // outside the window), and the time derivatives taken as the snapshots' secant slope
 // inside it.
-template <typename T, int POT = POT_RUNTIME>
+template <typename T, int POT = POT_RUNTIME, int EV = EV_OTHER>
 __device__ __forceinline__ void gather_td(const GridMeta<T> &gm, T x, T y, T z, T t_rel, Sample<T> &s)
 {
     Sample<T> s1;
-    gather<T, POT>(gm, x, y, z, s, &s1);
+    gather<T, POT, EV>(gm, x, y, z, s, &s1);
     // the window test on the time itself: at t_rel == span the weight may round above 1
     const bool inside = (t_rel >= T(0)) && (t_rel <= gm.span);
     T w = t_rel * gm.inv_span;
@@ -486,15 +501,15 @@ struct Aux {
 template <typename T>
 __device__ __forceinline__ void cross3(const T a[3], const T b[3], T c[3])
 {
-    c[0] = a[1] * b[2] - a[2] * b[1];
-    c[1] = a[2] * b[0] - a[0] * b[2];
-    c[2] = a[0] * b[1] - a[1] * b[0];
+    c[0] = m_fma(a[1], b[2], -m_mul(a[2], b[1]));
+    c[1] = m_fma(a[2], b[0], -m_mul(a[0], b[2]));
+    c[2] = m_fma(a[0], b[1], -m_mul(a[1], b[0]));
 }
 
 template <typename T>
 __device__ __forceinline__ T dot3(const T a[3], const T b[3])
 {
-    return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+    return m_fma(a[2], b[2], m_fma(a[0], b[0], m_mul(a[1], b[1])));
 }
 
 // J w for the channel block dF (J_cj = sum_d dF[d][c] g[d][j]) given p_d = g[d].w
@@ -555,14 +570,14 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
     T sb[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d)
-        sb[d] = s.dB[d][0] * b[0] + s.dB[d][1] * b[1] + s.dB[d][2] * b[2];
+        sb[d] = m_fma(s.dB[d][2], b[2], m_fma(s.dB[d][0], b[0], m_mul(s.dB[d][1], b[1])));
     // the grid's phi-index gradient has no z component (g[2][2] = 0)
     constexpr bool kGridG = POT != POT_RUNTIME;
     T gB[3];
 #pragma unroll
     for (int jx = 0; jx < 3; ++jx)
-        gB[jx] = (kGridG && jx == 2) ? sb[0] * s.g[0][2] + sb[1] * s.g[1][2]
-                                     : sb[0] * s.g[0][jx] + sb[1] * s.g[1][jx] + sb[2] * s.g[2][jx];
+        gB[jx] = (kGridG && jx == 2) ? m_fma(sb[0], s.g[0][2], m_mul(sb[1], s.g[1][2]))
+                                     : m_fma(sb[2], s.g[2][jx], m_fma(sb[0], s.g[0][jx], m_mul(sb[1], s.g[1][jx])));
     const T b_gB = dot3(b, gB);
 
     // E x B drift
@@ -586,7 +601,7 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
         Epar = ideal ? T(0) : dot3(s.E, b);
     }
     // gamma^2 = 1 + (gamma v)^2 / c^2 with (gamma v)^2 = u^2 + 2 mu_B B / m
-    const T g2 = T(1) + (u * u + T(2) * mub * Bm * ph.inv_m) * ph.inv_c2;
+    const T g2 = m_fma(m_fma(u, u, m_mul(T(2) * mub * Bm, ph.inv_m)), ph.inv_c2, T(1));
     const T inv_g = m_rsqrt(g2);
     const T gamma = g2 * inv_g;
     const T vpar = u * inv_g;
@@ -607,11 +622,11 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
         T wv[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            wv[c] = vpar * b[c] + vE[c];
+            wv[c] = m_fma(vpar, b[c], vE[c]);
         T pw[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d)
-            pw[d] = (kGridG && d == 2) ? s.g[2][0] * wv[0] + s.g[2][1] * wv[1] : dot3(s.g[d], wv);
+            pw[d] = (kGridG && d == 2) ? m_fma(s.g[2][0], wv[0], m_mul(s.g[2][1], wv[1])) : dot3(s.g[d], wv);
         T JBw[3], JEw[3];
         jvec2(s.dB, s.dE, pw, JBw, JEw);
         const T w_gB = dot3(wv, gB);
@@ -619,14 +634,14 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
         T wgb[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            wgb[c] = (JBw[c] - b[c] * w_gB) * inv_B;
+            wgb[c] = m_mul(m_fma(-b[c], w_gB, JBw[c]), inv_B);
         // (w.grad)v_E = ((J_E w) x B + E x (J_B w)) / B^2 - 2 v_E (w.grad|B|) / |B|
         T t1[3], t2[3], wgv[3];
         cross3(JEw, s.B, t1);
         cross3(s.E, JBw, t2);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            wgv[c] = (t1[c] + t2[c]) * inv_B2 - T(2) * vE[c] * w_gB * inv_B;
+            wgv[c] = m_fma(m_add(t1[c], t2[c]), inv_B2, -m_mul(m_mul(m_mul(T(2), vE[c]), w_gB), inv_B));
 
         // Eq. 1 bracket
         const T c_gB = mub * ph.inv_m * inv_g * inv_g;
@@ -634,7 +649,7 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
         if constexpr (POT == POT_IDEAL) {
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-                br[c] = c_gB * gB[c] + vpar * wgb[c] + wgv[c];
+                br[c] = m_add(m_fma(c_gB, gB[c], m_mul(vpar, wgb[c])), wgv[c]);
         } else {
             const T c_vE = ph.qm * vpar * Epar * ph.inv_c2 * inv_g;
 #pragma unroll
@@ -661,14 +676,14 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
         const T pre = gamma * inv_B * ph.inv_qm;
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            F[c] = vpar * b[c] + vE[c] + pre * bxbr[c];
+            F[c] = m_fma(pre, bxbr[c], wv[c]);
         // Eq. 2
         T w2[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
             w2[c] = wgb[c] + dbdt[c];
         if constexpr (POT == POT_IDEAL)
-            F[3] = gamma * dot3(vE, w2) - mub * ph.inv_m * inv_g * b_gB;
+            F[3] = m_fma(gamma, dot3(vE, w2), -m_mul(mub * ph.inv_m * inv_g, b_gB));
         else
             F[3] = ph.qm * Epar - mub * ph.inv_m * inv_g * b_gB + gamma * dot3(vE, w2);
     }
@@ -680,15 +695,15 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
         aux.b[c] = b[c];
 }
 
-template <typename T, bool TD = false, int POT = POT_RUNTIME>
+template <typename T, bool TD = false, int POT = POT_RUNTIME, int EV = EV_OTHER>
 __device__ __forceinline__ uint32_t eval_F(const GridMeta<T> &gm, const Phys<T> &ph, T x, T y, T z,
                                            T u, T mub, T F[4], Aux<T> &aux, T t_rel = T(0))
 {
     Sample<T> s;
     if constexpr (TD)
-        gather_td<T, POT>(gm, x, y, z, t_rel, s);
+        gather_td<T, POT, EV>(gm, x, y, z, t_rel, s);
     else
-        gather<T, POT>(gm, x, y, z, s);
+        gather<T, POT, EV>(gm, x, y, z, s);
     rhs<T, TD, POT>(s, ph, gm.ideal, u, mub, F, aux);
     return s.flags;
 }

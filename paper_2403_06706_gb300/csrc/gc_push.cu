@@ -13,6 +13,8 @@
 // field and Eqs. 1-2 in float and accumulates R, gamma v_par and the free path in
 // double-float pairs; mu_B is a double-float too (the right-hand side takes its float
 // part), and the rare collision and rebirth updates of gamma v_par and mu_B run in double.
+#include <type_traits>
+
 #include "gc_push.cuh"
 
 namespace gcp {
@@ -103,24 +105,25 @@ __global__ void __launch_bounds__((kPushThreads<T, TD>), 1) push_kernel(const __
             int n_phase = 2;
             // phase 0: predictor point and corrector; phase 1: F^{n+1}, free path, events;
             // after an event, phases 2-3 restart the history out of line
-            auto run_phase = [&](int phase) {
+            auto run_phase = [&](auto kind, int phase) {
+                constexpr int EV = decltype(kind)::value;
                 T px, py, pz, pu;
                 phase_point(phase, s, w, dtT, px, py, pz, pu);
                 T Fo[4];
                 Aux<T> ax;
-                s.flags |= eval_F<T, TD, POT>(gm, ph, px, py, pz, pu, s.mub, Fo, ax,
+                s.flags |= eval_F<T, TD, POT, EV>(gm, ph, px, py, pz, pu, s.mub, Fo, ax,
                                               phase == 3 ? t_end - dtT : t_end);
                 phase_consume(phase, n_phase, i, s, c, Fo, ax, w, P, ph, dtT, t0, (long long)(P.kbase + k + 1),
                               n_coll, n_reb);
             };
+            using std::integral_constant;
             if constexpr (kUnrollPhases) {
-#pragma unroll
-                for (int phase = 0; phase < 2; ++phase)
-                    run_phase(phase);
+                run_phase(integral_constant<int, EV_PREDICTOR>{}, 0);
+                run_phase(integral_constant<int, EV_CORRECTOR>{}, 1);
             } else {
 #pragma unroll 1
                 for (int phase = 0; phase < 2; ++phase)
-                    run_phase(phase);
+                    run_phase(integral_constant<int, EV_PREDICTOR>{}, phase);
             }
             if (n_phase == 4) {
                 using Acc = AccOf<T>;

@@ -372,15 +372,15 @@ __device__ __forceinline__ void phase_point(int phase, const PState<T> &s, const
     pz = Acc::val(s.Rz);
     pu = Acc::val(s.U);
     if (phase == 0) {
-        px += w.a0 * s.F0[0] + w.a1 * s.F1[0];
-        py += w.a0 * s.F0[1] + w.a1 * s.F1[1];
-        pz += w.a0 * s.F0[2] + w.a1 * s.F1[2];
-        pu += w.a0 * s.F0[3] + w.a1 * s.F1[3];
+        px = m_add(px, m_fma(w.a0, s.F0[0], m_mul(w.a1, s.F1[0])));
+        py = m_add(py, m_fma(w.a0, s.F0[1], m_mul(w.a1, s.F1[1])));
+        pz = m_add(pz, m_fma(w.a0, s.F0[2], m_mul(w.a1, s.F1[2])));
+        pu = m_add(pu, m_fma(w.a0, s.F0[3], m_mul(w.a1, s.F1[3])));
     } else if (phase == 3) {
-        px -= dtT * s.F0[0];
-        py -= dtT * s.F0[1];
-        pz -= dtT * s.F0[2];
-        pu -= dtT * s.F0[3];
+        px = m_fma(-dtT, s.F0[0], px);
+        py = m_fma(-dtT, s.F0[1], py);
+        pz = m_fma(-dtT, s.F0[2], pz);
+        pu = m_fma(-dtT, s.F0[3], pu);
     }
 }
 
@@ -513,10 +513,10 @@ __device__ __forceinline__ void phase_consume(int phase, int &n_phase, int64_t i
 {
     using Acc = AccOf<T>;
     if (phase == 0) {
-        s.Rx = Acc::add(s.Rx, w.c0 * s.F0[0] + w.cs * Fo[0] + w.c1 * s.F1[0]);
-        s.Ry = Acc::add(s.Ry, w.c0 * s.F0[1] + w.cs * Fo[1] + w.c1 * s.F1[1]);
-        s.Rz = Acc::add(s.Rz, w.c0 * s.F0[2] + w.cs * Fo[2] + w.c1 * s.F1[2]);
-        s.U = Acc::add(s.U, w.c0 * s.F0[3] + w.cs * Fo[3] + w.c1 * s.F1[3]);
+        s.Rx = Acc::add(s.Rx, m_fma(w.c1, s.F1[0], m_fma(w.c0, s.F0[0], m_mul(w.cs, Fo[0]))));
+        s.Ry = Acc::add(s.Ry, m_fma(w.c1, s.F1[1], m_fma(w.c0, s.F0[1], m_mul(w.cs, Fo[1]))));
+        s.Rz = Acc::add(s.Rz, m_fma(w.c1, s.F1[2], m_fma(w.c0, s.F0[2], m_mul(w.cs, Fo[2]))));
+        s.U = Acc::add(s.U, m_fma(w.c1, s.F1[3], m_fma(w.c0, s.F0[3], m_mul(w.cs, Fo[3]))));
     } else if (phase == 1) {
         const T px = Acc::val(s.Rx), py = Acc::val(s.Ry), pz = Acc::val(s.Rz);
         // Sect. 2.3: path length along B in this step
