@@ -180,7 +180,8 @@ __device__ __forceinline__ void polar_angles(double x, double y, double z, doubl
 }
 
 // The evaluations of a step associate the two radii's sums differently (as the FP32 push's
-// results have had them): EV_OTHER stands for injections, restarts and field samples.
+// results have had them): EV_OTHER stands for injections and field samples, and `other` at run
+// time for the restarts among a step's evaluations.
 enum : int { EV_OTHER = 0, EV_PREDICTOR, EV_CORRECTOR };
 
 // ----------------------------------------------------------------------------------------
@@ -388,15 +389,18 @@ __device__ __forceinline__ void interp_nodes(const T *__restrict__ nodes, uint32
 // the interpolant is extended as a constant.
 template <typename T, int POT = POT_RUNTIME, int EV = EV_OTHER>
 __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sample<T> &s,
-                                       Sample<T> *s1 = nullptr)
+                                       Sample<T> *s1 = nullptr, bool other = false)
 {
     uint32_t flags = 0;
+    other = other || EV == EV_OTHER;
     T rho2 = EV == EV_OTHER ? m_fma(x, x, m_mul(y, y)) : m_fma(y, y, m_mul(x, x));
+    if (EV != EV_OTHER && __builtin_expect(other, 0))
+        rho2 = m_fma(x, x, m_mul(y, y));
     if (!(rho2 > T(1e-30))) {
         flags |= FLAG_AXIS;
         rho2 = T(1e-30);
     }
-    const T r2 = EV == EV_CORRECTOR && POT != POT_ON ? m_add(rho2, m_mul(z, z)) : m_fma(z, z, rho2);
+    const T r2 = EV == EV_CORRECTOR && POT != POT_ON && !other ? m_add(rho2, m_mul(z, z)) : m_fma(z, z, rho2);
     const T inv_rho = m_rsqrt(rho2), inv_r = m_rsqrt(r2);
     const T rho = rho2 * inv_rho, r = r2 * inv_r;
     T theta, phi;
@@ -456,10 +460,11 @@ __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sam
 // outside the window), and the time derivatives taken as the snapshots' secant slope
 // inside it.
 template <typename T, int POT = POT_RUNTIME, int EV = EV_OTHER>
-__device__ __forceinline__ void gather_td(const GridMeta<T> &gm, T x, T y, T z, T t_rel, Sample<T> &s)
+__device__ __forceinline__ void gather_td(const GridMeta<T> &gm, T x, T y, T z, T t_rel, Sample<T> &s,
+                                          bool other = false)
 {
     Sample<T> s1;
-    gather<T, POT, EV>(gm, x, y, z, s, &s1);
+    gather<T, POT, EV>(gm, x, y, z, s, &s1, other);
     // the window test on the time itself: at t_rel == span the weight may round above 1
     const bool inside = (t_rel >= T(0)) && (t_rel <= gm.span);
     T w = t_rel * gm.inv_span;
@@ -697,13 +702,13 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
 
 template <typename T, bool TD = false, int POT = POT_RUNTIME, int EV = EV_OTHER>
 __device__ __forceinline__ uint32_t eval_F(const GridMeta<T> &gm, const Phys<T> &ph, T x, T y, T z,
-                                           T u, T mub, T F[4], Aux<T> &aux, T t_rel = T(0))
+                                           T u, T mub, T F[4], Aux<T> &aux, T t_rel = T(0), bool other = false)
 {
     Sample<T> s;
     if constexpr (TD)
-        gather_td<T, POT, EV>(gm, x, y, z, t_rel, s);
+        gather_td<T, POT, EV>(gm, x, y, z, t_rel, s, other);
     else
-        gather<T, POT, EV>(gm, x, y, z, s);
+        gather<T, POT, EV>(gm, x, y, z, s, nullptr, other);
     rhs<T, TD, POT>(s, ph, gm.ideal, u, mub, F, aux);
     return s.flags;
 }
