@@ -97,6 +97,14 @@ __device__ __forceinline__ float m_sqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ double m_sqrt(double a) { return sqrt(a); }
 __device__ __forceinline__ float m_rsqrt(float a) { return rsqrtf(a); }
 __device__ __forceinline__ double m_rsqrt(double a) { return rsqrt(a); }
+// the same for a normal argument: without the range scaling of the general FP32 form
+__device__ __forceinline__ float m_rsqrt_normal(float a)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ double m_rsqrt_normal(double a) { return rsqrt(a); }
 __device__ __forceinline__ float m_floor(float a) { return floorf(a); }
 __device__ __forceinline__ double m_floor(double a) { return floor(a); }
 __device__ __forceinline__ float m_rcp(float a) { return __fdividef(1.0f, a); }
@@ -124,11 +132,16 @@ template <> __device__ __forceinline__ double two_pi<double>() { return 6.283185
 // p of degree 7 fitted for minimal maximum error on [0, 1] (|error| < 4e-8 for the fitted
 // coefficients, < 7.1e-8 at t = 1 with them rounded to the float literals below; the fit is
 // reproduced by csrc/atan_coeffs.py), then unfold the octant.
-__device__ __forceinline__ float m_atan2(float y, float x)
+// POS: y > 0 is known (the polar angle), its sign and the point (0, 0) need no care.
+template <bool POS>
+__device__ __forceinline__ float m_atan2_t(float y, float x)
 {
-    const float ax = fabsf(x), ay = fabsf(y);
+    const float ax = fabsf(x), ay = POS ? y : fabsf(y);
     const float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
-    const float t = mx > 0.0f ? __fdividef(mn, mx) : 0.0f;
+    // flushing form: the general one scales its operands, for quotients below 2^-126 only
+    float t;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(t) : "f"(mn), "f"(mx));
+    if (!POS) t = mx > 0.0f ? t : 0.0f;
     const float s = t * t;
     float p = -4.059181749e-03f;
     p = fmaf(p, s, 2.188265529e-02f);
@@ -141,8 +154,9 @@ __device__ __forceinline__ float m_atan2(float y, float x)
     float r = t * p;
     if (ay > ax) r = 1.57079632679489662f - r;
     if (x < 0.0f) r = 3.14159265358979324f - r;
-    return copysignf(r, y);
+    return POS ? r : copysignf(r, y);
 }
+__device__ __forceinline__ float m_atan2(float y, float x) { return m_atan2_t<false>(y, x); }
 
 // FP64 polar angle of (X, Y) given inv_h = 1 / hypot(X, Y) and an FP32 estimate `est` of
 // the angle (within 1e-6 rad), without a double-precision atan2. Take the reference angle
@@ -169,7 +183,7 @@ __device__ __forceinline__ double refine_angle(double X, double Y, double inv_h,
 __device__ __forceinline__ void polar_angles(float x, float y, float z, float rho, float, float,
                                              float &theta, float &phi)
 {
-    theta = m_atan2(rho, z);
+    theta = m_atan2_t<true>(rho, z);
     phi = m_atan2(y, x);
 }
 __device__ __forceinline__ void polar_angles(double x, double y, double z, double rho, double inv_rho,
@@ -401,7 +415,7 @@ __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sam
         rho2 = T(1e-30);
     }
     const T r2 = EV == EV_CORRECTOR && POT != POT_ON && !other ? m_add(rho2, m_mul(z, z)) : m_fma(z, z, rho2);
-    const T inv_rho = m_rsqrt(rho2), inv_r = m_rsqrt(r2);
+    const T inv_rho = m_rsqrt_normal(rho2), inv_r = m_rsqrt_normal(r2);
     const T rho = rho2 * inv_rho, r = r2 * inv_r;
     T theta, phi;
     polar_angles(x, y, z, rho, inv_rho, inv_r, theta, phi);
@@ -410,28 +424,28 @@ __device__ __forceinline__ void gather(const GridMeta<T> &gm, T x, T y, T z, Sam
     T xr = m_mul(m_fma(r2, inv_r, -gm.r_min), gm.inv_dr);
     T xt = theta * gm.inv_dth;
     T xp = phi * gm.inv_dph;
-    if (!(m_finite(xr) && m_finite(xt) && m_finite(xp))) {
+    if (!m_finite(xr + xt + xp)) { // one test: none of them comes near the largest float
         flags |= FLAG_NONFINITE;
         xr = T(0); xt = T(0); xp = T(0);
     }
-    if (xr < T(-1) || xr > T(gm.n_r))
-        flags |= FLAG_OUT_OF_GRID;
 
     const T flr = m_floor(xr);
     int i = (int)flr;
     T fr = m_sub(xr, flr);
-    if (i < 0) { i = 0; fr = T(0); }
-    else if (i > gm.n_r - 2) { i = gm.n_r - 2; fr = T(1); }
+    if (__builtin_expect((unsigned)i > (unsigned)(gm.n_r - 2), 0)) { // outside the shell's cells: rare
+        if (xr < T(-1) || xr > T(gm.n_r))
+            flags |= FLAG_OUT_OF_GRID;
+        fr = i < 0 ? T(0) : T(1);
+        i = i < 0 ? 0 : gm.n_r - 2;
+    }
     const T flt = m_floor(xt);
     int j = (int)flt;
     T ft = m_sub(xt, flt);
-    if (j < 0) { j = 0; ft = T(0); }
-    else if (j > gm.n_th - 2) { j = gm.n_th - 2; ft = T(1); }
+    if (j > gm.n_th - 2) { j = gm.n_th - 2; ft = T(1); } // theta >= 0
     const T flp = m_floor(xp);
     int k = (int)flp;
     const T fp = m_sub(xp, flp);
-    if (k >= gm.n_ph) k -= gm.n_ph;
-    if (k < 0) k += gm.n_ph;
+    if (k >= gm.n_ph) k -= gm.n_ph; // phi in [0, 2 pi]
     const int k1 = (k + 1 == gm.n_ph) ? 0 : k + 1;
 
     const uint32_t nr8 = (uint32_t)gm.n_r * 8u;
@@ -607,7 +621,7 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
     }
     // gamma^2 = 1 + (gamma v)^2 / c^2 with (gamma v)^2 = u^2 + 2 mu_B B / m
     const T g2 = m_fma(m_fma(u, u, m_mul(T(2) * mub * Bm, ph.inv_m)), ph.inv_c2, T(1));
-    const T inv_g = m_rsqrt(g2);
+    const T inv_g = m_rsqrt_normal(g2); // g2 >= 1
     const T gamma = g2 * inv_g;
     const T vpar = u * inv_g;
 
