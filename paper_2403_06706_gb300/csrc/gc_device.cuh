@@ -154,7 +154,8 @@ __device__ __forceinline__ float m_atan2_t(float y, float x)
     float r = t * p;
     if (ay > ax) r = 1.57079632679489662f - r;
     if (x < 0.0f) r = 3.14159265358979324f - r;
-    return POS ? r : copysignf(r, y);
+    if (POS) return r;
+    return copysignf(r, y);
 }
 __device__ __forceinline__ float m_atan2(float y, float x) { return m_atan2_t<false>(y, x); }
 
