@@ -426,6 +426,8 @@ int enqueue_advance(gc_ctx *c, cudaStream_t s, double dt, int64_t n_steps, doubl
     P.clock = clock_dev;
     P.spread_from = INT64_MAX;
     if (c->grid_waves == 1) gcp::push_spread(P, block, grid);
+    // a launch shape that was asked for is kept
+    const bool quad = c->block == 0 && c->grid_waves == 1 && gcp::push_quad_fits(c->opt.precision, c->gh, c->n, c->sm_count);
     const gcp::PhysHost ph = c->phys();
 
     int64_t done = 0;
@@ -443,7 +445,10 @@ int enqueue_advance(gc_ctx *c, cudaStream_t s, double dt, int64_t n_steps, doubl
         Timed t;
         TRY(new_interval(c, 0, owned, &t));
         CUDA_TRY(cudaEventRecord(t.a, s));
-        CUDA_TRY(gcp::launch_push(c->opt.precision, c->gh, ph, P, block, grid, s));
+        if (quad)
+            CUDA_TRY(gcp::launch_push_quad(c->gh, ph, P, s));
+        else
+            CUDA_TRY(gcp::launch_push(c->opt.precision, c->gh, ph, P, block, grid, s));
         CUDA_TRY(cudaEventRecord(t.b, s));
         lc->kernels += 1;
         lc->pushes += 1;

@@ -532,16 +532,8 @@ __device__ __forceinline__ T dot3(const T a[3], const T b[3])
     return m_fma(a[2], b[2], m_fma(a[0], b[0], m_mul(a[1], b[1])));
 }
 
-// J w for the channel block dF (J_cj = sum_d dF[d][c] g[d][j]) given p_d = g[d].w
-template <typename T>
-__device__ __forceinline__ void jvec(const T dF[3][3], const T p[3], T out[3])
-{
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        out[c] = dF[0][c] * p[0] + dF[1][c] * p[1] + dF[2][c] * p[2];
-}
-
-// J_B p and J_E p together; FP32: the six channels as three packed pairs (Bx By | Bz Ex |
+// J w for the channel blocks dB and dE (J_cj = sum_d dF[d][c] g[d][j]) given p_d = g[d].w;
+// FP32: the six channels as three packed pairs (Bx By | Bz Ex |
 // Ey Ez), the pairs the gather interpolated, two FMAs per instruction
 template <typename T>
 __device__ __forceinline__ void jvec2(const T dB[3][3], const T dE[3][3], const T p[3], T JB[3], T JE[3])
@@ -568,8 +560,11 @@ __device__ __forceinline__ void jvec2(const T dB[3][3], const T dE[3][3], const 
         p2_split(acc[1], JB[2], JE[0]);
         p2_split(acc[2], JE[1], JE[2]);
     } else {
-        jvec(dB, p, JB);
-        jvec(dE, p, JE);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            JB[c] = m_fma(dB[2][c], p[2], m_fma(dB[0][c], p[0], m_mul(dB[1][c], p[1])));
+            JE[c] = m_fma(dE[2][c], p[2], m_fma(dE[0][c], p[0], m_mul(dE[1][c], p[1])));
+        }
     }
 }
 
@@ -616,7 +611,10 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
 #pragma unroll
         for (int d = 0; d < 3; ++d)
             pb[d] = dot3(s.g[d], b);
-        Epar = -(s.dPhi[0] * pb[0] + s.dPhi[1] * pb[1] + s.dPhi[2] * pb[2]);
+        if constexpr (sizeof(T) == 8)
+            Epar = -dot3(s.dPhi, pb);
+        else
+            Epar = -(s.dPhi[0] * pb[0] + s.dPhi[1] * pb[1] + s.dPhi[2] * pb[2]);
     } else {
         Epar = ideal ? T(0) : dot3(s.E, b);
     }
@@ -632,6 +630,8 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
             F[c] = vpar * b[c];
         if constexpr (POT == POT_IDEAL)
             F[3] = -(mub * ph.inv_m * inv_g * b_gB);
+        else if constexpr (sizeof(T) == 8)
+            F[3] = m_fma(ph.qm, Epar, -m_mul(mub * ph.inv_m * inv_g, b_gB));
         else
             F[3] = ph.qm * Epar - mub * ph.inv_m * inv_g * b_gB;
     } else {
@@ -674,7 +674,8 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
             const T c_vE = ph.qm * vpar * Epar * ph.inv_c2 * inv_g;
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-                br[c] = c_gB * gB[c] + c_vE * vE[c] + vpar * wgb[c] + wgv[c];
+                br[c] = sizeof(T) == 8 ? m_add(m_fma(c_vE, vE[c], m_fma(c_gB, gB[c], m_mul(vpar, wgb[c]))), wgv[c])
+                                       : c_gB * gB[c] + c_vE * vE[c] + vpar * wgb[c] + wgv[c];
         }
         // time-dependent fields: v_par db/dt + dv_E/dt in the bracket, and db/dt in Eq. 2's
         // v_E product, with db/dt = (dB/dt - b (b.dB/dt)) / B and
@@ -704,6 +705,8 @@ __device__ __forceinline__ void rhs(const Sample<T> &s, const Phys<T> &ph, int i
             w2[c] = wgb[c] + dbdt[c];
         if constexpr (POT == POT_IDEAL)
             F[3] = m_fma(gamma, dot3(vE, w2), -m_mul(mub * ph.inv_m * inv_g, b_gB));
+        else if constexpr (sizeof(T) == 8)
+            F[3] = m_fma(gamma, dot3(vE, w2), m_fma(ph.qm, Epar, -m_mul(mub * ph.inv_m * inv_g, b_gB)));
         else
             F[3] = ph.qm * Epar - mub * ph.inv_m * inv_g * b_gB + gamma * dot3(vE, w2);
     }

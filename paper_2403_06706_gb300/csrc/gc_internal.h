@@ -115,6 +115,9 @@ cudaError_t launch_push(int precision, const GridHost &g, const PhysHost &ph, co
                         int block, int grid, cudaStream_t s);
 cudaError_t launch_inject(int precision, const GridHost &g, const PhysHost &ph,
                           const InjectParams &p, cudaStream_t s);
+// the FP64 push of few particles, four lanes each: whether it applies, and its launch
+bool push_quad_fits(int precision, const GridHost &g, int64_t n, int sms);
+cudaError_t launch_push_quad(const GridHost &g, const PhysHost &ph, const PushParams &p, cudaStream_t s);
 // set the spread of the last round for a grid of one resident wave (p.st.n is set)
 void push_spread(PushParams &p, int block, int grid);
 // most threads per block of the push, as many as an SM holds of it

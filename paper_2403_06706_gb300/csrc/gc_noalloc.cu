@@ -253,13 +253,15 @@ extern "C" int gc_advance_noalloc(const gc_options *opt, const gc_grid_desc *g, 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, opt->device);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((sd->n + 31) / 32, (int64_t)sms * nb));
     gcp::push_spread(P, block, grid);
+    const bool quad = gcp::push_quad_fits(opt->precision, gh, sd->n, sms);
     int64_t done = 0;
     while (sd->n > 0 && done < n_steps) {
         const int64_t chunk = std::min<int64_t>(n_steps - done, 2000);
         P.step0 = step0 + done;
         P.kbase = done;
         P.n_steps = (int32_t)chunk;
-        if ((e = gcp::launch_push(opt->precision, gh, ph, P, block, grid, s)) != cudaSuccess)
+        e = quad ? gcp::launch_push_quad(gh, ph, P, s) : gcp::launch_push(opt->precision, gh, ph, P, block, grid, s);
+        if (e != cudaSuccess)
             return nfail(GC_ERR_CUDA, "gc_advance_noalloc: launch: %s", cudaGetErrorString(e));
         done += chunk;
     }

@@ -157,6 +157,323 @@ __global__ void __launch_bounds__((kPushThreads<T, TD>), 1) push_kernel(const __
 }
 
 // ----------------------------------------------------------------------------------------
+// FP64 push of a small population: four lanes per particle. An FP64 instruction holds its
+// scheduler's pipe for 64 cycles whatever the number of active lanes, so with fewer particles
+// than lanes the time is the number of instructions in a particle's chain, which spreading the
+// particles thinner does not shorten. Lane c = 0, 1, 2 of a quad holds component c of every
+// vector (and the channels B_c, E_c of the gather), lane 3 gamma v_par and the potential;
+// products over components and cross products go through shuffles, the polar angles and the
+// roots of the two radii are taken in different lanes at once, scalars are carried by all four.
+// Rounding for rounding what push_kernel does, so that the launch's shape and the size of the
+// population don't show in the results. 400 steps, E_par = 0, one particle per lane -> this:
+// 608 to 2432 particles 10.15 -> 5.9 ms, 4864 6.3 ms, 7296 8.4, 9728 10.9 (from four warps
+// per SM on the pipe is shared, and the work common to the lanes counts): push_quad_fits.
+__device__ __forceinline__ double q_get(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 4); }
+
+// dot3 of two vectors held by lanes 0-2: the chain of its three roundings goes round the lanes
+__device__ __forceinline__ double q_dot(double a, double b)
+{
+    double t = a * b;
+    t = m_fma(a, b, q_get(t, 1));
+    t = m_fma(a, b, q_get(t, 0));
+    return q_get(t, 2);
+}
+
+// component c of cross3: a1, a2 and b1, b2 are the next two components
+__device__ __forceinline__ double q_cross(double a1, double a2, double b1, double b2) { return m_fma(a1, b2, -m_mul(a2, b1)); }
+
+struct QuadEval {
+    double F;           // this lane's component of (F_x, F_y, F_z, F_u)
+    double vpar, Bm, b; // b: this lane's component
+    double r2;          // squared radius of the point
+    uint32_t flags;
+};
+
+// Eqs. 1-3 at the point whose component (x, y, z, gamma v_par) this lane holds in p: gather and
+// rhs, rounding for rounding
+template <int POT, int EV>
+__device__ __forceinline__ QuadEval quad_eval(const GridMeta<double> &gm, const Phys<double> &ph, int c, double p, double mub,
+                                              bool other)
+{
+    QuadEval o;
+    const int c1 = (c + 1) % 3, c2 = (c + 2) % 3; // the next components, cyclically (lane 3: any)
+    const double x = q_get(p, 0), y = q_get(p, 1), z = q_get(p, 2), u = q_get(p, 3);
+    uint32_t flags = 0;
+    double rho2 = other ? m_fma(x, x, m_mul(y, y)) : m_fma(y, y, m_mul(x, x));
+    if (!(rho2 > 1e-30)) {
+        flags |= FLAG_AXIS;
+        rho2 = 1e-30;
+    }
+    const double r2 = EV == EV_CORRECTOR && POT != POT_ON && !other ? m_add(rho2, m_mul(z, z)) : m_fma(z, z, rho2);
+    const double inv = m_rsqrt(c == 0 ? rho2 : r2);
+    const double inv_rho = q_get(inv, 0), inv_r = q_get(inv, 1);
+    const double rho = rho2 * inv_rho;
+    // index coordinates: lane 0 theta, lane 1 phi, lane 2 r
+    const double X = c == 0 ? z : x, Y = c == 0 ? rho : y;
+    double ang = refine_angle(X, Y, c == 0 ? inv_r : inv_rho, m_atan2((float)Y, (float)X));
+    if (c == 1 && ang < 0.0) ang += two_pi<double>();
+    double q = c == 2 ? m_mul(m_fma(r2, inv_r, -gm.r_min), gm.inv_dr) : ang * (c == 0 ? gm.inv_dth : gm.inv_dph);
+    const unsigned lane0 = threadIdx.x & 28u;
+    if ((__ballot_sync(0xffffffffu, !m_finite(q)) >> lane0) & 7u) {
+        flags |= FLAG_NONFINITE;
+        q = 0.0;
+    }
+    const double fl = floor(q);
+    int idx = (int)fl;
+    double f = q - fl;
+    const int last = c == 2 ? gm.n_r - 2 : gm.n_th - 2;
+    const bool out = c == 2 && (q < -1.0 || q > gm.n_r);
+    if ((__ballot_sync(0xffffffffu, out) >> lane0) & 4u) flags |= FLAG_OUT_OF_GRID;
+    if (c == 1) {
+        if (idx >= gm.n_ph) idx -= gm.n_ph;
+    } else if (idx < 0 || idx > last) {
+        f = idx < 0 ? 0.0 : 1.0;
+        idx = idx < 0 ? 0 : last;
+    }
+    const int i = __shfl_sync(0xffffffffu, idx, 2, 4), j = __shfl_sync(0xffffffffu, idx, 0, 4),
+              k = __shfl_sync(0xffffffffu, idx, 1, 4);
+    const double fr = q_get(f, 2), ft = q_get(f, 0), fp = q_get(f, 1);
+    const int kn = k + 1 == gm.n_ph ? 0 : k + 1;
+
+    // channels B_c and E_c (lane 3: the potential, and E_x unused)
+    const uint32_t nr8 = (uint32_t)gm.n_r * 8u;
+    const uint32_t o0 = (((uint32_t)k * (uint32_t)gm.n_th + (uint32_t)j) * (uint32_t)gm.n_r + (uint32_t)i) * 8u;
+    const uint32_t o1 = (((uint32_t)kn * (uint32_t)gm.n_th + (uint32_t)j) * (uint32_t)gm.n_r + (uint32_t)i) * 8u;
+    double val[2], d[2][3];
+#pragma unroll
+    for (int ch = 0; ch < 2; ++ch) {
+        const double *nodes = gm.nodes + (ch == 0 ? (c < 3 ? c : 7) : 3 + (c < 3 ? c : 0));
+        double L[2][2], D[2][2];
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const double *n0 = nodes + (cc ? o1 : o0) + (b ? nr8 : 0u);
+                const double v0 = __ldg(n0), v1 = __ldg(n0 + 8);
+                D[b][cc] = v1 - v0;
+                L[b][cc] = v0 + fr * D[b][cc];
+            }
+        double V[2], Dr[2], Dt[2];
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+            Dt[cc] = L[1][cc] - L[0][cc];
+            V[cc] = L[0][cc] + ft * Dt[cc];
+            Dr[cc] = D[0][cc] + ft * (D[1][cc] - D[0][cc]);
+        }
+        d[ch][2] = V[1] - V[0];
+        val[ch] = V[0] + fp * d[ch][2];
+        d[ch][0] = Dr[0] + fp * (Dr[1] - Dr[0]);
+        d[ch][1] = Dt[0] + fp * (Dt[1] - Dt[0]);
+    }
+    const double B = val[0], E = val[1];
+    // this lane's component of the index coordinates' gradients (see gather)
+    const double st = inv_r * inv_r * gm.inv_dth, sp = inv_rho * inv_rho * gm.inv_dph;
+    double g[3];
+    g[0] = p * (inv_r * gm.inv_dr);
+    g[1] = (c < 2 ? z * inv_rho * p : -rho) * st;
+    g[2] = c == 0 ? -y * sp : (c == 1 ? x * sp : 0.0);
+
+    // the right-hand side
+    const double B2 = q_dot(B, B);
+    const double inv_B = m_rsqrt(B2), Bm = B2 * inv_B, inv_B2 = inv_B * inv_B, b = B * inv_B;
+    double sb[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        sb[a] = q_dot(d[0][a], b);
+    const double gB01 = m_fma(sb[0], g[0], m_mul(sb[1], g[1]));
+    const double gB = c == 2 ? gB01 : m_fma(sb[2], g[2], gB01);
+    const double b_gB = q_dot(b, gB);
+    const double B1 = q_get(B, c1), Bq = q_get(B, c2), E1 = q_get(E, c1), Eq = q_get(E, c2);
+    const double vE = q_cross(E1, Eq, B1, Bq) * inv_B2;
+    double Epar = 0.0;
+    if constexpr (POT == POT_ON) {
+        double pb[3], dPhi[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            pb[a] = q_dot(g[a], b);
+            dPhi[a] = q_get(d[0][a], 3);
+        }
+        Epar = -dot3(dPhi, pb);
+    } else if constexpr (POT == POT_NONE) {
+        Epar = q_dot(E, b);
+    }
+    const double g2 = m_fma(m_fma(u, u, m_mul(2.0 * mub * Bm, ph.inv_m)), ph.inv_c2, 1.0);
+    const double inv_g = m_rsqrt(g2), gamma = g2 * inv_g, vpar = u * inv_g;
+    const double mirror = m_mul(mub * ph.inv_m * inv_g, b_gB);
+    double F, Fu;
+    if (ph.drift_mask == 1) {
+        F = vpar * b;
+        Fu = POT == POT_IDEAL ? -mirror : m_fma(ph.qm, Epar, -mirror);
+    } else {
+        const double wv = m_fma(vpar, b, vE);
+        double pw[3];
+        pw[0] = q_dot(g[0], wv);
+        pw[1] = q_dot(g[1], wv);
+        pw[2] = q_get(m_fma(g[2], wv, q_get(m_mul(g[2], wv), 1)), 0);
+        const double JB = m_fma(d[0][2], pw[2], m_fma(d[0][0], pw[0], m_mul(d[0][1], pw[1])));
+        const double JE = m_fma(d[1][2], pw[2], m_fma(d[1][0], pw[0], m_mul(d[1][1], pw[1])));
+        const double w_gB = q_dot(wv, gB);
+        const double wgb = m_mul(m_fma(-b, w_gB, JB), inv_B);
+        const double t1 = q_cross(q_get(JE, c1), q_get(JE, c2), B1, Bq);
+        const double t2 = q_cross(E1, Eq, q_get(JB, c1), q_get(JB, c2));
+        const double wgv = m_fma(m_add(t1, t2), inv_B2, -m_mul(m_mul(m_mul(2.0, vE), w_gB), inv_B));
+        double br = m_fma(mub * ph.inv_m * inv_g * inv_g, gB, m_mul(vpar, wgb));
+        if constexpr (POT != POT_IDEAL) br = m_fma(ph.qm * vpar * Epar * ph.inv_c2 * inv_g, vE, br);
+        br = m_add(br, wgv);
+        const double bxbr = q_cross(q_get(b, c1), q_get(b, c2), q_get(br, c1), q_get(br, c2));
+        F = m_fma(gamma * inv_B * ph.inv_qm, bxbr, wv);
+        const double vw = q_dot(vE, wgb);
+        Fu = m_fma(gamma, vw, POT == POT_IDEAL ? -mirror : m_fma(ph.qm, Epar, -mirror));
+    }
+    o.F = c == 3 ? Fu : F;
+    o.vpar = vpar;
+    o.Bm = Bm;
+    o.b = b;
+    o.r2 = r2;
+    o.flags = flags;
+    return o;
+}
+
+template <int POT>
+__global__ void __launch_bounds__(32, 1) push_quad_kernel(const __grid_constant__ GridMeta<double> gm,
+                                                       const __grid_constant__ Phys<double> ph,
+                                                       const __grid_constant__ PushParams P)
+{
+    const int lane = threadIdx.x & 31, c = lane & 3;
+    const unsigned quad = 0xFu << (lane & 28);
+    const int64_t slot = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+    // quads past the end shadow the last particle, so that whole warps shuffle
+    const bool real = slot < P.st.n;
+    const int64_t i = real ? slot : P.st.n - 1, cap = P.st.cap;
+    const double dt = P.dt;
+    double t0 = P.t0;
+    int64_t step0 = P.step0;
+    if (P.clock) {
+        t0 = P.clock[0];
+        step0 = (int64_t)P.clock[1] + P.kbase;
+    }
+    const StepW<double> w1 = {dt * 1.5, dt * -0.5, dt * (2.0 / 3.0), dt * (5.0 / 12.0), dt * (-1.0 / 12.0)};
+    const uint32_t e = P.st.ens[i];
+    // squared radii beyond which the shell's test is due, a rounding inside the shell
+    const double r_in2 = P.ens[e].r_in > 0.0 ? P.ens[e].r_in * P.ens[e].r_in * (1.0 + 1e-14) : 0.0;
+    const double r_out2 = P.ens[e].r_out > 0.0 ? P.ens[e].r_out * P.ens[e].r_out * (1.0 - 1e-14) : 0.0;
+    double *const own = c == 0 ? P.st.x : (c == 1 ? P.st.y : (c == 2 ? P.st.z : P.st.u));
+    double A = own[i], F0 = P.st.F0[c * cap + i], F1 = P.st.F1[c * cap + i];
+    double S = P.st.s_rem[i], mub = P.st.mub[i], vpar0 = P.st.vpar[i], hprev = P.st.h_prev[i];
+    double t_birth = P.st.t_birth[i], Bm0 = 0.0;
+    uint32_t event = P.st.event[i], ncoll = P.st.ncoll[i], flags = P.st.flags[i];
+    unsigned n_coll = 0, n_reb = 0;
+
+    int next_tally = INT32_MAX - 1;
+    if (P.tally_on) {
+        const int64_t K = P.tally.cadence;
+        next_tally = (int)((K - 1 - (step0 % K)) % K);
+    }
+    int k = 0;
+    do {
+        const int k_end = min(P.n_steps, next_tally + 1);
+        bool restart = false;
+        // as in push_kernel: a restarting particle spends an iteration on its start-up history;
+        // quads that are through evaluate on without effect until the warp's last is
+        while (__any_sync(0xffffffffu, k < k_end)) {
+            const bool act = k < k_end;
+            const StepW<double> w = step_weights(w1, dt, hprev);
+            const QuadEval a = quad_eval<POT, EV_PREDICTOR>(gm, ph, c, m_add(A, m_fma(w.a0, F0, m_mul(w.a1, F1))), mub, restart);
+            if (act) {
+                flags |= a.flags;
+                if (restart) {
+                    F0 = a.F;
+                    vpar0 = a.vpar;
+                    Bm0 = a.Bm;
+                } else {
+                    A += m_fma(w.c1, F1, m_fma(w.c0, F0, m_mul(w.cs, a.F)));
+                }
+            }
+            const QuadEval o = quad_eval<POT, EV_CORRECTOR>(gm, ph, c, restart ? m_fma(-dt, F0, A) : A, mub, restart);
+            if (!act) continue;
+            flags |= o.flags;
+            if (restart) {
+                F1 = o.F;
+                restart = false;
+            } else {
+                // Sect. 2.3: path length along B in this step
+                const double ds = dt * (fabs(vpar0) + fabs(o.vpar)) * 0.5;
+                bool collide = false;
+                if (!P.no_scatter) {
+                    if (P.collision_form == 0) {
+                        S -= ds;
+                        collide = S <= 0.0;
+                    } else {
+                        const uint4 wd = draw(P.st.id[i], P.seed, event++);
+                        collide = u53(wd.x, wd.y) < 1.0 - exp(-ds / lambda_of(P, P.ens[e]));
+                    }
+                }
+                auto at = [&](double v, int src) { return __shfl_sync(quad, v, src, 4); };
+                bool reborn = false;
+                if (!P.no_rebirth && (o.r2 < r_in2 || o.r2 > r_out2)) {
+                    const double xx = at(A, 0), yy = at(A, 1), zz = at(A, 2);
+                    const double r1 = sqrt(xx * xx + yy * yy + zz * zz);
+                    reborn = r1 < P.ens[e].r_in || r1 > P.ens[e].r_out;
+                }
+                if (reborn || collide) {
+                    RareState<double> s{at(A, 0), at(A, 1), at(A, 2), at(A, 3), S, mub, t_birth, event, ncoll};
+                    s = rare_event<double>(P, ph, i, reborn, s, o.Bm, at(o.b, 0), at(o.b, 1), at(o.b, 2), t0,
+                                           (long long)(P.kbase + k + 1));
+                    A = c == 0 ? s.Rx : (c == 1 ? s.Ry : (c == 2 ? s.Rz : s.U));
+                    S = s.S;
+                    mub = s.mub;
+                    t_birth = s.t_birth;
+                    event = s.event;
+                    ncoll = s.ncoll;
+                    if (real && c == 0) {
+                        if (reborn)
+                            ++n_reb;
+                        else
+                            ++n_coll;
+                    }
+                    F0 = F1 = 0.0;
+                    restart = true;
+                    continue;
+                }
+                F1 = F0;
+                F0 = o.F;
+                vpar0 = o.vpar;
+                Bm0 = o.Bm;
+            }
+            hprev = dt;
+            ++k;
+        }
+        if (k == next_tally + 1) {
+            next_tally += P.tally.cadence;
+            const double x = q_get(A, 0), y = q_get(A, 1), z = q_get(A, 2), u = q_get(A, 3);
+            const double t_new = step_time(t0, (long long)(P.kbase + k), P.dt);
+            tally_sample<double>(P.tally, P, ph, e, x, y, z, u, mub, Bm0, t_new - t_birth, ncoll,
+                                 real && c == 0 && t_birth >= P.tally.t_start && (int)e < P.tally.n_ens);
+        }
+    } while (k < P.n_steps);
+
+    // what the last step leaves (see push_kernel); lanes of components x, u and x's F^n
+    const unsigned bad = __ballot_sync(0xffffffffu, !m_finite(A) || (c == 0 && !m_finite(F0)));
+    if ((bad >> (lane & 28)) & 9u) flags |= FLAG_NONFINITE;
+    if (real) {
+        own[i] = A;
+        P.st.F0[c * cap + i] = F0;
+        P.st.F1[c * cap + i] = F1;
+        if (c == 0) {
+            P.st.s_rem[i] = S;
+            P.st.mub[i] = mub;
+            P.st.vpar[i] = vpar0;
+            P.st.h_prev[i] = hprev;
+            P.st.t_birth[i] = t_birth;
+            P.st.event[i] = event;
+            P.st.ncoll[i] = ncoll;
+            store_flags(P, i, flags);
+        }
+    }
+    flush_counters(P, n_coll, n_reb);
+}
+
+// ----------------------------------------------------------------------------------------
 // Injection (Sect. 3): site, mu0 and energy draws (Philox events 0 and 1), start-up history.
 struct InjDraw {
     double mu0, pm; // pitch cosine and momentum magnitude |p| / m = gamma v
@@ -451,6 +768,22 @@ InjectFn<T> inject_fn(bool td, bool pot)
     return pot ? inject_kernel<T, false, POT_ON> : inject_kernel<T, false, POT_NONE>;
 }
 
+// FP64, a steady field, and at most six warps of quads per SM (8.4 ms instead of 10.2; with
+// eight 10.9)
+bool push_quad_fits(int precision, const GridHost &g, int64_t n, int sms)
+{
+    return precision == 0 && !g.nodes1 && n > 0 && n <= (int64_t)sms * 48;
+}
+
+cudaError_t launch_push_quad(const GridHost &g, const PhysHost &ph, const PushParams &p, cudaStream_t s)
+{
+    cudaGetLastError(); // report this launch only
+    const int grid = (int)((p.st.n + 7) / 8);
+    const auto fn = g.ideal == 2 ? push_quad_kernel<POT_ON> : (g.ideal == 1 ? push_quad_kernel<POT_IDEAL> : push_quad_kernel<POT_NONE>);
+    fn<<<grid, 32, 0, s>>>(make_meta<double>(g), make_phys<double>(ph), p);
+    return cudaGetLastError();
+}
+
 int push_threads(int precision, bool time_dependent)
 {
     if (precision == 0) return time_dependent ? kPushThreads<double, true> : kPushThreads<double, false>;
@@ -531,6 +864,9 @@ cudaError_t preload_kernels()
         e = cudaFuncGetAttributes(&a, push_fn<float>(v & 1, v & 2, v & 4));
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, push_fn<double>(v & 1, v & 2, v & 4));
     }
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, push_quad_kernel<POT_ON>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, push_quad_kernel<POT_IDEAL>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, push_quad_kernel<POT_NONE>);
     return e;
 }
 
