@@ -31,7 +31,7 @@ sys.path.insert(0, ROOT)
 
 from paper_2403_06706_gb300 import synth  # noqa: E402
 
-LAUNCH = dict(block=128, steps_per_launch=1000, sort_every=1000)
+LAUNCH = dict(steps_per_launch=1000, sort_every=1000)  # the library's own launch shape
 PUSH_STEPS = 1000
 TALLY = dict(cadence=100, n_mu=32, n_E=32, n_r=64, n_age=32, E_lo_keV=5.0, E_hi_keV=600.0,
              r_lo_au=0.1, r_hi_au=2.5, age_max_s=86400.0, rwin_lo_au=0.9, rwin_hi_au=1.1,
@@ -58,7 +58,7 @@ FP64_PEAK_NOMINAL_TFLOPS = 1.25  # nominal dense FP64 of a GB300
 # ncu counters of the push kernels (DRAM bytes of one launch, thread instructions per
 # particle-step, FP64 pipe activity), with the sha256 of the kernel sources they were taken on
 COUNTERS_FILE = os.path.join(ROOT, "profiles", "push_counters.txt")
-COUNTER_SOURCES = ("gc_push.cu", "gc_device.cuh", "gc_internal.h", "unit_circle_table.h")
+COUNTER_SOURCES = ("gc_push.cu", "gc_push.cuh", "gc_device.cuh", "gc_f32x2.cuh", "gc_internal.h", "unit_circle_table.h")
 SM_REASONS = ("hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap")
 # Neural field: tensor-core work of one evaluation with its Jacobian (value + 3 tangent
 # rows through three 256 x 256 layers and the 256 x 8 output layer, FMA = 2 flop)

@@ -1,7 +1,7 @@
 // gc_push.cu -- persistent guiding-centre push and injection kernels (sm_103a).
 //
-// One thread owns one particle at a time and keeps its whole state in registers for all
-// the steps of a launch (grid-stride over particles). Per step (Sect. 2.2):
+// One thread (in FP64, for few particles, four lanes) owns one particle at a time and keeps its
+// whole state in registers for all the steps of a launch. Per step (Sect. 2.2):
 //   predictor X* (Eq. 5) -> F* = F(X*) -> corrector X^{n+1} (Eq. 6) -> F^{n+1}
 //   -> free path decrement by dt (|v_par^n| + |v_par^{n+1}|)/2 (Sect. 2.3, Eq. 9)
 //   -> rebirth if the particle left [r_in, r_out], else a collision if the free path is

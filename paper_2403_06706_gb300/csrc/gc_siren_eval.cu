@@ -6,7 +6,8 @@
 //   layer 1:  z = w0 (W1 x + b1),   h1 = sin z,   t1_j = w0 cos(z) W1[:, j]
 //   layer k:  z = W_k h_{k-1} + b_k, h_k = sin z, t_{k,j} = cos(z) * (W_k t_{k-1,j})
 //   output:   y = W5 h4 + b5,       J[:, j] = W5 t_{4,j}.
-// A tile is 64 points = 256 rows (row 4p + q: q = 0 value, q = 1..3 tangents). Hidden
+// A tile is 64 points = 256 rows (row 4p + q: q = 0 value, q = 1..3 tangents), or 16 points =
+// 64 rows where that leaves every SM at most one tile (kSmallTiles). Hidden
 // layers run as D = W_k . H^T on the tensor cores (two halves of M = 128 output features,
 // N = 256 rows, K = 256), so that each accumulator lane holds one feature and the four rows
 // of a point sit in adjacent columns: the epilogue thread of a feature computes sin and cos
@@ -32,7 +33,7 @@
 //
 // Warp roles (576 threads): warps 0-15 compute; all of them work on one output half at a
 // time, warp w on features 32 (w % 4) + lane of the half (warp w may only touch
-// tensor-memory lanes 32 (w % 4) .. + 31) and rows 64 (w / 4) .. + 63. Warp 16 lane 0 issues the MMAs
+// tensor-memory lanes 32 (w % 4) .. + 31) and rows 64 (w / 4) .. + 63. One lane of warp 16 issues the MMAs
 // (warp 16 also owns the tensor-memory allocation), warp 17 lane 0 issues the TMA loads.
 // Every wait is bounded: a wait that runs out sets the kernel's error word and an abort flag
 // that makes all roles leave their loops; the CTA then waits for its own copies and MMAs

@@ -21,7 +21,7 @@
 // What bounds kernel 1: the tile is one dependent chain of 13 steps, about 48 000 cycles, of
 // which the CUDA cores' own work (sine and cosine of 4 x 256 pre-activations per sample at
 // library accuracy, dW5) is about 30 000 and the tensor cores' 10 000 (a 128 x 64 x 16 MMA
-// takes 48 cycles: shared memory). 210 us of 292 us for loss and gradient of 65536 samples;
+// takes 48 cycles: shared memory). 210 us of 270 us for loss and gradient of 65536 samples;
 // kernel 2 takes 42 us, reading 300 MB at 7 TB/s. Before, each layer made passes over
 // [sample][256] buffers (FP32 pre-activations, their gradients: 2 GB of traffic): 905 us.
 // Warp roles of kernel 1 (608 threads): warps 0-15 compute (warp w: features 32 (w % 4) +
@@ -50,6 +50,14 @@ constexpr uint32_t kBoxBytes = 128u * 128u;    // one TMA box of weights: 128 ro
 constexpr uint32_t kStageBytes = 2 * kBoxBytes; // 128 x 128 weights
 constexpr uint32_t kActBytes = 256u * 128u;    // 256 features x 64 samples bf16
 constexpr uint32_t kW5Bytes = 4u * 16u * 128u; // W5 padded to 16 rows: 4 boxes of 16 x 64
+// Samples of a batch up to which sine and cosine are the library's, one value at a time. The
+// fast ones differ from them in the last place; where that moves a BF16 rounding, everything
+// behind it in the sample is rounded anew, and the gradient moves by 8e-4 / sqrt(samples):
+// 3.5e-5 for 512, 4e-6 for 32768 (either is 2e-3 from the gradient in FP64, BF16's rounding).
+// So that small batches, which are bound by the chain's latency, take the same roundings as
+// plain sinf and cosf: within 1.3e-6. At 512 samples 71 us for loss and gradient (215 with
+// a pass over memory per layer), at 16384 132 (395), at 32768 with the fast ones 169 (541).
+constexpr int64_t kLibrarySines = 16384;
 constexpr int kStagesPerTile = 24;             // 6 products x 4
 constexpr int kComputeThreads = 512;
 constexpr int kThreads = 608;
@@ -110,8 +118,8 @@ __device__ __forceinline__ void load_rows16(const uint8_t *frow, uint32_t rsw, i
     }
 }
 
-// Sine and / or cosine of 16 values (in place where an output is the input). Beyond the fast
-// reduction's range the library's, one value at a time and out of line: pre-activations of a
+// Sine and / or cosine of 16 values (in place where an output is the input). With LIB, and
+// beyond the fast reduction's range, the library's, one value at a time and out of line: pre-activations of a
 // trained network stay below about 10^2.
 __device__ __noinline__ float2 sincos_any(float z)
 {
@@ -120,14 +128,14 @@ __device__ __noinline__ float2 sincos_any(float z)
     return make_float2(s, c);
 }
 
-template <bool SIN, bool COS>
+template <bool LIB, bool SIN, bool COS>
 __device__ __forceinline__ void sincos16(const float (&z)[16], float (&sn)[16], float (&cs)[16])
 {
     float m = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; ++i)
         m = fmaxf(m, fabsf(z[i]));
-    if (m <= gcp::kSincosMax) {
+    if (!LIB && m <= gcp::kSincosMax) {
 #pragma unroll
         for (int i = 0; i < 16; i += 2) {
             float s[2], c[2];
@@ -145,6 +153,7 @@ __device__ __forceinline__ void sincos16(const float (&z)[16], float (&sn)[16], 
     }
 }
 
+template <bool LIB>
 __global__ void __launch_bounds__(kThreads, 1)
     siren_train_kernel(const __grid_constant__ CUtensorMap mwh, const __grid_constant__ CUtensorMap mw5, const __grid_constant__ CUtensorMap mact,
                        const __grid_constant__ TrainParams p)
@@ -418,7 +427,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float4 q = wpts[i];
                     v[i] = w0 * fmaf(wa, q.x, fmaf(wb, q.y, fmaf(wc, q.z, b1)));
                 }
-                sincos16<true, false>(v, o, v);
+                sincos16<LIB, true, false>(v, o, v);
                 store_rows16(sAct[0] + frow + h * (kActBytes / 2), rsw, rg, o);
                 announce(h);
             }
@@ -438,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int i = 0; i < 16; ++i)
                         v[i] += b;
                     float c[16];
-                    sincos16<true, true>(v, o, c);
+                    sincos16<LIB, true, true>(v, o, c);
                     store_rows16(sAct[buf] + frow + h * (kActBytes / 2), rsw, rg, o);
                     tmem_st16(ta, c);
                     announce(h);
@@ -553,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float4 q = wpts[i];
                     c[i] = w0 * fmaf(wa, q.x, fmaf(wb, q.y, fmaf(wc, q.z, b1)));
                 }
-                sincos16<false, true>(c, v, c);
+                sincos16<LIB, false, true>(c, v, c);
                 if (!wait_acc(h)) { ok = false; break; }
                 tmem_ld16(lane_base + region(0) + h * 64, v);
 #pragma unroll
@@ -728,8 +737,8 @@ cudaError_t train_fwd_bwd(const SirenNet &net, const CUtensorMap &act, const flo
 {
     if (n <= 0) return cudaSuccess;
     if (n % kRows != 0 || !net.err) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(siren_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemTrain);
+    const auto fn = n <= kLibrarySines ? siren_train_kernel<true> : siren_train_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTrain);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(train_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDw);
     if (e != cudaSuccess) return e;
@@ -746,8 +755,7 @@ cudaError_t train_fwd_bwd(const SirenNet &net, const CUtensorMap &act, const flo
     p.loss = loss;
     p.err = net.err;
     const int64_t tiles = n / kRows;
-    siren_train_kernel<<<(int)(tiles < sms ? tiles : sms), kThreads, kSmemTrain, s>>>(net.map_wh, net.map_w5,
-                                                                                     act, p);
+    fn<<<(int)(tiles < sms ? tiles : sms), kThreads, kSmemTrain, s>>>(net.map_wh, net.map_w5, act, p);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // 6 CTAs (3 layers x 2 halves) per split of the batch: as many splits as fill the SMs once

@@ -1,7 +1,9 @@
 """The fused training pass (loss and gradient) at the edges of its tiling, against the oracle's
 BF16 reading: two 64-sample tiles; two tiles more than the 152 CTAs of a launch; several tiles
-per CTA with a ragged last round. Bounds as for one batch in test_gpu_siren.py (FP32 summation
-order and the BF16 rounding flips it causes). The last case has first-layer arguments on both
+per CTA with a ragged last round; the last batch that takes the library's sines and the first
+that takes the fast ones. Bounds as for one batch in test_gpu_siren.py (FP32 summation
+order and the BF16 rounding flips it causes). The cases at
+omega0 = 4e4 have first-layer arguments on both
 sides of the fast sine's range (|z| <= 30000): there FP32 itself leaves z uncertain by three
 roundings of 2^-24 |z|, 7e-3 rad at 4e4, in every h1, so the gradient is held to 5e-2 (an
 argument sent through the wrong reduction would leave nothing of it)."""
@@ -17,7 +19,8 @@ torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("n,omega0,tol", [(128, 30.0, 2e-3), (154 * 64, 30.0, 2e-3), (458 * 64, 30.0, 2e-3),
-                                          (1024, 4.0e4, 5e-2)])
+                                          (1024, 4.0e4, 5e-2), (16384, 30.0, 2e-3), (16512, 30.0, 2e-3),
+                                          (16512, 4.0e4, 5e-2)])
 def test_gradient_at_tile_edges(n, omega0, tol):
     rng = np.random.default_rng(n)
     p = synth.siren_init(seed=n)
