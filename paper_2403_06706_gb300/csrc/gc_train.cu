@@ -119,8 +119,8 @@ __device__ __forceinline__ void load_rows16(const uint8_t *frow, uint32_t rsw, i
 }
 
 // Sine and / or cosine of 16 values (in place where an output is the input). With LIB, and
-// beyond the fast reduction's range, the library's, one value at a time and out of line: pre-activations of a
-// trained network stay below about 10^2.
+// beyond the fast reduction's range, the library's, one value at a time and out of line:
+// pre-activations of a trained network stay below about 10^2.
 __device__ __noinline__ float2 sincos_any(float z)
 {
     float s, c;

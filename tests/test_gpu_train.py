@@ -2,9 +2,9 @@
 BF16 reading: two 64-sample tiles; two tiles more than the 152 CTAs of a launch; several tiles
 per CTA with a ragged last round; the last batch that takes the library's sines and the first
 that takes the fast ones. Bounds as for one batch in test_gpu_siren.py (FP32 summation
-order and the BF16 rounding flips it causes). The cases at
-omega0 = 4e4 have first-layer arguments on both
-sides of the fast sine's range (|z| <= 30000): there FP32 itself leaves z uncertain by three
+order and the BF16 rounding flips it causes). The cases at omega0 = 4e4 have first-layer
+arguments on both sides of the fast sine's range (|z| <= 30000): there FP32 itself leaves z
+uncertain by three
 roundings of 2^-24 |z|, 7e-3 rad at 4e4, in every h1, so the gradient is held to 5e-2 (an
 argument sent through the wrong reduction would leave nothing of it)."""
 import numpy as np
