@@ -21,8 +21,8 @@
 // What bounds kernel 1: the tile is one dependent chain of 13 steps, about 48 000 cycles, of
 // which the CUDA cores' own work (sine and cosine of 4 x 256 pre-activations per sample at
 // library accuracy, dW5) is about 30 000 and the tensor cores' 10 000 (a 128 x 64 x 16 MMA
-// takes 48 cycles: shared memory). 210 us of 270 us for loss and gradient of 65536 samples;
-// kernel 2 takes 42 us, reading 300 MB at 7 TB/s. Before, each layer made passes over
+// takes 48 cycles: shared memory). 203 us of 270 us for loss and gradient of 65536 samples;
+// kernel 2 takes 41 us, reading 300 MB, two thirds of them from memory. Before, each layer made passes over
 // [sample][256] buffers (FP32 pre-activations, their gradients: 2 GB of traffic): 905 us.
 // Warp roles of kernel 1 (608 threads): warps 0-15 compute (warp w: features 32 (w % 4) +
 // lane of a half, samples 16 (w / 4) ..), warp 16 issues MMAs, warp 17 TMA loads of the
