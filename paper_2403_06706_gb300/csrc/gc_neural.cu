@@ -104,10 +104,11 @@ __device__ __forceinline__ void target_point(const T *__restrict__ nodes, const 
     double ft = xt - j;
     if (j < 0) { j = 0; ft = 0; }
     else if (j > g.n_th - 2) { j = g.n_th - 2; ft = 1; }
-    int k = (int)floor(xp);
+    // a NaN (whose conversion is the lowest integer) reads the first cell and leaves a NaN in fp;
+    // in r and theta the clamps above catch it
+    int k = xp >= 0 ? (int)floor(xp) : 0;
     const double fp = xp - k;
     if (k >= g.n_ph) k -= g.n_ph;
-    if (k < 0) k += g.n_ph;
     const int k1 = (k + 1 == g.n_ph) ? 0 : k + 1;
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int a = 0; a < 2; ++a)

@@ -76,3 +76,27 @@ def test_targets_are_the_rounded_interpolant():
         err = np.abs(t - to) / (2.0**-24 * np.abs(to) * 1.0001 + 1e-10 * scale + 1e-45)
         print(err.max(0))
         assert err.max() <= 1.0
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_targets_of_points_that_are_no_numbers(dtype):
+    """A NaN coordinate gives NaN targets (the potential's may stay a number where only z is
+    one) and reads inside the grid; infinities are beyond the shell. The points beside them
+    have the targets that they have alone."""
+    w = synth.WindSpec(17, 9, 12, eps=0.1, n_modes=2, phi1_v=100.0)
+    x = np.random.default_rng(1).uniform(-0.5, 0.5, (300, 3)).astype(np.float32)
+    nan, inf = np.nan, np.inf
+    x[100:109] = [[nan, 0.3, 0.2], [0.3, nan, 0.2], [0.3, 0.2, nan], [nan, nan, 0.1], [nan, nan, nan],
+                  [inf, nan, 0.1], [inf, 0.1, 0.1], [-inf, -inf, inf], [nan, 0.0, -inf]]
+    good = np.r_[:100, 109:300]
+    with gcpush.Context(precision=gcpush.PREC_FP64 if dtype == np.float64 else gcpush.PREC_FP32_MIXED) as c:
+        c.field_load(synth.wind_grid(w, dtype=dtype), w.r_min_au, w.r_max_au)
+        c.siren_set(synth.siren_init(0), r_max_au=w.r_max_au, B_scale=w.B1, E_scale=w.B1 * w.u_sw)
+        t = torch.zeros((300, 8), device="cuda")
+        c.field_targets(torch.from_numpy(x).cuda(), t)
+        alone = torch.zeros((len(good), 8), device="cuda")
+        c.field_targets(torch.from_numpy(x[good]).cuda(), alone)
+    t, alone = t.cpu().numpy(), alone.cpu().numpy()
+    assert np.isnan(t[100:106, :7]).all() and np.isnan(t[108, :7]).all()
+    assert np.isnan(t[[100, 101, 103, 104, 105, 108], 7]).all()
+    assert np.isfinite(alone).all() and np.array_equal(t[good], alone)
