@@ -469,10 +469,16 @@ cudaError_t neural_targets(const Neural &nn, const GridRef &g, const float *x, i
 
 cudaError_t neural_loss_grad(Neural &nn, const float *x, const float *t, int64_t n, float *grad, cudaStream_t s)
 {
-    float *g = grad ? grad : nn.G;
-    cudaError_t e = cudaMemsetAsync(g, 0, (size_t)kSirenNParams * sizeof(float), s);
+    // train_dw_kernel adds groups of four floats: a gradient that is not aligned for them (a slice
+    // of a caller's flat buffer) is summed in the network's own and copied out
+    const bool direct = grad && ((uintptr_t)grad & 15u) == 0;
+    float *g = direct ? grad : nn.G;
+    const size_t bytes = (size_t)kSirenNParams * sizeof(float);
+    cudaError_t e = cudaMemsetAsync(g, 0, bytes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(&nn.d_status->loss, 0, sizeof(double), s);
-    return e == cudaSuccess ? fwd_bwd(nn, x, t, n, g, s) : e;
+    if (e == cudaSuccess) e = fwd_bwd(nn, x, t, n, g, s);
+    if (e == cudaSuccess && grad && !direct) e = cudaMemcpyAsync(grad, g, bytes, cudaMemcpyDeviceToDevice, s);
+    return e;
 }
 
 cudaError_t neural_status_copy(Neural &nn, cudaStream_t s)

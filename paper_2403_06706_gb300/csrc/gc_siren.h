@@ -72,7 +72,7 @@ bool siren_push_fits(int64_t n);
 cudaError_t siren_push(const SirenNet &net, const SirenIn &in, const SirenOut &out, const gcp::PhysHost &phys,
                        const gcp::PushParams &push, int ideal, cudaStream_t s);
 // Training (gc_train.cu): adds the gradient of the mean squared error of n samples (n a
-// multiple of 64) to G and the sum of squared residuals to loss. act: tensor map, made by
+// multiple of 64) to G (16-byte aligned) and the sum of squared residuals to loss. act: tensor map, made by
 // train_act_map, of a BF16 work buffer of 6 x 256 rows of `cap` >= n samples (h1..h3, dz2..dz4).
 cudaError_t train_act_map(CUtensorMap *m, const void *act, int64_t cap);
 cudaError_t train_fwd_bwd(const SirenNet &net, const CUtensorMap &act, const float *x, const float *t, int64_t n,

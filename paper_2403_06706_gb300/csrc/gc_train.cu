@@ -736,7 +736,7 @@ cudaError_t train_fwd_bwd(const SirenNet &net, const CUtensorMap &act, const flo
                           float *G, double *loss, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    if (n % kRows != 0 || !net.err) return cudaErrorInvalidValue;
+    if (n % kRows != 0 || !net.err || ((uintptr_t)G & 15u) != 0) return cudaErrorInvalidValue;
     const auto fn = n <= kLibrarySines ? siren_train_kernel<true> : siren_train_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTrain);
     if (e == cudaSuccess)

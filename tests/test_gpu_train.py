@@ -100,3 +100,25 @@ def test_targets_of_points_that_are_no_numbers(dtype):
     assert np.isnan(t[100:106, :7]).all() and np.isnan(t[108, :7]).all()
     assert np.isnan(t[[100, 101, 103, 104, 105, 108], 7]).all()
     assert np.isfinite(alone).all() and np.array_equal(t[good], alone)
+
+
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_gradient_into_a_slice_of_a_flat_buffer(off):
+    """A gradient buffer at 4-byte alignment gets the aligned one's gradient and nothing beside
+    it is written. The two differ by the order of FP32 atomics alone: up to two tiles x four
+    row groups are added per parameter, 7 roundings of at most 2^-24 of the terms' sum, held to
+    1e-5 of the gradient's norm."""
+    n = 128
+    rng = np.random.default_rng(off)
+    x = torch.from_numpy(rng.uniform(-0.6, 0.6, (n, 3)).astype(np.float32)).cuda()
+    t = torch.from_numpy((rng.normal(size=(n, 8)) * 0.3).astype(np.float32)).cuda()
+    flat = torch.full((gcpush.SIREN_NPARAMS + 8,), 7.0, device="cuda")
+    view = flat[off:off + gcpush.SIREN_NPARAMS]
+    g = torch.empty(gcpush.SIREN_NPARAMS, device="cuda")
+    assert view.data_ptr() % 16 != 0 and g.data_ptr() % 16 == 0
+    with gcpush.Context() as c:
+        c.siren_set(synth.siren_init(seed=1), omega0=30.0)
+        loss = c.siren_loss_grad(x, t, g)
+        assert abs(c.siren_loss_grad(x, t, view) - loss) < 1e-12 * loss
+    assert float((view - g).norm()) < 1e-5 * float(g.norm()) > 0.0
+    assert bool((flat[:off] == 7.0).all()) and bool((flat[off + gcpush.SIREN_NPARAMS:] == 7.0).all())
