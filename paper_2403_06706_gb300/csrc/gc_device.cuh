@@ -138,10 +138,13 @@ __device__ __forceinline__ float m_atan2_t(float y, float x)
 {
     const float ax = fabsf(x), ay = POS ? y : fabsf(y);
     const float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
-    // flushing form: the general one scales its operands, for quotients below 2^-126 only
+    // Flushing form: the general one scales its operands, for quotients below 2^-126 and
+    // subnormal operands only. A subnormal mn counts as zero, and with the smallest normal float
+    // as the least denominator so does 0 / 0, whether mx is zero or subnormal: a point next to
+    // the axis has the longitude of the nearer axis (exact ones there, by a branch that scales
+    // the operands, cost 2 % of the push, and the nodes of a pole are one point).
     float t;
-    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(t) : "f"(mn), "f"(mx));
-    if (!POS) t = mx > 0.0f ? t : 0.0f;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(t) : "f"(mn), "f"(POS ? mx : fmaxf(mx, 1.17549435e-38f)));
     const float s = t * t;
     float p = -4.059181749e-03f;
     p = fmaf(p, s, 2.188265529e-02f);
