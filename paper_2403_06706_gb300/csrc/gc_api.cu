@@ -377,24 +377,25 @@ int blocks_per_sm(gc_ctx *c, int block)
     return nb;
 }
 
-// Threads per block of the push: what gc_set_launch or the autotuner chose, else one block per
-// SM (FP32 of 934 000 particles 2.88e10 particle-steps/s with blocks of 128, 2.91e10 of 256,
-// 2.99e10 of 512; two-fluid field and wind 2.14e10, 2.17e10, 2.25e10).
+// Threads per block of the push: what gc_set_launch or the autotuner chose, else the library's
+// own shape.
 int push_block(gc_ctx *c)
 {
-    return c->block ? c->block : gcp::push_threads(c->opt.precision, c->gh.nodes1 != nullptr);
+    return c->block ? c->block : gcp::push_block(c->opt.precision, c->gh.nodes1 != nullptr, c->n, c->sm_count);
 }
 
 int push_grid(gc_ctx *c, int block)
 {
-    const int nb = blocks_per_sm(c, block);
     const int64_t want = (c->n + block - 1) / block;
     if (c->grid_waves <= 0)
         return (int)std::min<int64_t>(want, 0x7FFFFFFF);
+    // the library's own shape has one block per SM
+    const int nb = c->block || c->grid_waves > 1 ? blocks_per_sm(c, block) : 1;
     const int64_t wave = (int64_t)c->grid_waves * c->sm_count * nb;
-    // one wave is spread over all SMs (push_spread), down to 32 particles per block
+    // one wave is spread over all SMs (push_spread), down to one group of particles per block
     const bool spread = c->grid_waves == 1 && block % 128 == 0;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(spread ? (c->n + 31) / 32 : want, wave));
+    const int group = gcp::push_group(c->opt.precision);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(spread ? (c->n + group - 1) / group : want, wave));
 }
 
 // Enqueue the launches of one advance on stream s: cell sorts on schedule and push

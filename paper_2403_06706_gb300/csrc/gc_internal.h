@@ -120,8 +120,10 @@ bool push_quad_fits(int precision, const GridHost &g, int64_t n, int sms);
 cudaError_t launch_push_quad(const GridHost &g, const PhysHost &ph, const PushParams &p, cudaStream_t s);
 // set the spread of the last round for a grid of one resident wave (p.st.n is set)
 void push_spread(PushParams &p, int block, int grid);
-// most threads per block of the push, as many as an SM holds of it
-int push_threads(int precision, bool time_dependent);
+// threads per block of the library's own launch shape, one block per SM, for n particles
+int push_block(int precision, bool time_dependent, int64_t n, int sms);
+// particles of a partial round that a block takes at a time
+int push_group(int precision);
 int push_max_blocks_per_sm(int precision, int block, bool time_dependent = false, bool potential = false);
 // one split-step kernel (FP32 path) over n particles or list entries (at most)
 cudaError_t launch_split(int kind, const PhysHost &ph, const SplitParams &p, int64_t n, cudaStream_t s);

@@ -245,13 +245,11 @@ extern "C" int gc_advance_noalloc(const gc_options *opt, const gc_grid_desc *g, 
     P.gflags = d_flags;
     P.counters = d_counters;
 
-    const int block = gcp::push_threads(opt->precision, false); // one block per SM, as gc_advance
-    int nb = gcp::push_max_blocks_per_sm(opt->precision, block, false, g->ideal == 2);
-    cudaGetLastError(); // the occupancy query's status is not this call's
-    if (nb < 1) nb = 1;
+    // the launch shape of gc_advance: one block per SM
     int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, opt->device);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((sd->n + 31) / 32, (int64_t)sms * nb));
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, opt->device) != cudaSuccess || sms < 1) sms = 1;
+    const int block = gcp::push_block(opt->precision, false, sd->n, sms), group = gcp::push_group(opt->precision);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((sd->n + group - 1) / group, sms));
     gcp::push_spread(P, block, grid);
     const bool quad = gcp::push_quad_fits(opt->precision, gh, sd->n, sms);
     int64_t done = 0;

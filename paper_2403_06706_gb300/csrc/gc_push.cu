@@ -13,6 +13,7 @@
 // field and Eqs. 1-2 in float and accumulates R, gamma v_par and the free path in
 // double-float pairs; mu_B is a double-float too (the right-hand side takes its float
 // part), and the rare collision and rebirth updates of gamma v_par and mu_B run in double.
+#include <algorithm>
 #include <type_traits>
 
 #include "gc_push.cuh"
@@ -27,6 +28,10 @@ namespace gcp {
 // and 512 spill and measured 0.4 % and 1.7 % slower: the FP64 pipe, not latency, bounds it).
 template <typename T, bool TD>
 constexpr int kPushThreads = sizeof(T) == 4 ? (TD ? 384 : 512) : 256;
+
+// Particles of a partial round that a block takes at a time (see push_kernel).
+template <typename T>
+constexpr unsigned kSpread = sizeof(T) == 8 ? 32 : 128;
 
 // Fused push: one thread owns a particle for all the steps of a launch and evaluates the
 // grid field inline.
@@ -53,15 +58,15 @@ __global__ void __launch_bounds__((kPushThreads<T, TD>), 1) push_kernel(const __
     constexpr bool kUnrollPhases = !TD;
 
     // Particles of the full rounds in blocks of neighbours (which share cells); those left from
-    // P.spread_from on, all of a small population, in groups of kSpread, one per block in turn:
+    // P.spread_from on, all of a small population, in groups of kSpread<T>, one per block in turn:
     // a partial round then has its warps on all SMs. (With whole blocks 200 000 particles, 2.57
     // rounds of one block of 512 per SM, ran 11 % slower than with blocks of 128; groups of 32
     // instead of 128 3 % slower, but 8 % faster in FP64 where an SM gets fewer than four warps.)
-    constexpr unsigned kSpread = sizeof(T) == 8 ? 32 : 128;
+    constexpr unsigned group = kSpread<T>;
     int64_t next = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (;;) {
         if (next >= P.spread_from)
-            next = P.spread_from + ((int64_t)(threadIdx.x / kSpread) * gridDim.x + blockIdx.x) * kSpread + threadIdx.x % kSpread;
+            next = P.spread_from + ((int64_t)(threadIdx.x / group) * gridDim.x + blockIdx.x) * group + threadIdx.x % group;
         if (next >= P.st.n)
             break;
         const uint32_t i = (uint32_t)next; // ids, and so slots, have 32 bits
@@ -784,10 +789,24 @@ cudaError_t launch_push_quad(const GridHost &g, const PhysHost &ph, const PushPa
     return cudaGetLastError();
 }
 
-int push_threads(int precision, bool time_dependent)
+static int push_threads(int precision, bool time_dependent)
 {
     if (precision == 0) return time_dependent ? kPushThreads<double, true> : kPushThreads<double, false>;
     return time_dependent ? kPushThreads<float, true> : kPushThreads<float, false>;
+}
+
+int push_group(int precision) { return (int)(precision == 0 ? kSpread<double> : kSpread<float>); }
+
+// One block per SM that holds all the threads the registers allow (FP32 of 934 000 particles
+// 2.88e10 particle-steps/s with blocks of 128, 2.91e10 of 256, 2.99e10 of 512; two-fluid field and
+// wind 2.14e10, 2.17e10, 2.25e10), or as many as the particles need: a block keeps its registers
+// until its last thread is through, and what a small push does not use is there for another
+// context's (four of 19 456 particles on their own streams, 20 000 steps: 96 ms in blocks of 512,
+// 49 of 128; one alone 24 either way, and no size from 1000 to 160 000 takes longer).
+int push_block(int precision, bool time_dependent, int64_t n, int sms)
+{
+    const int64_t per_sm = (n + sms - 1) / sms;
+    return (int)std::max<int64_t>(128, std::min<int64_t>((per_sm + 127) / 128 * 128, push_threads(precision, time_dependent)));
 }
 
 void push_spread(PushParams &p, int block, int grid)

@@ -1,0 +1,66 @@
+"""The push's own launch shape for populations that do not fill the SMs: a block has as many
+threads as the population needs, so that several contexts' pushes run side by side, and no
+particle is lost or advanced twice at the edges between block sizes."""
+import threading
+import time
+
+import numpy as np
+import pytest
+
+from paper_2403_06706_gb300 import synth
+from test_gpu_spread import WIND, _run
+
+pytestmark = pytest.mark.gpu
+gcpush = pytest.importorskip("paper_2403_06706_gb300.gcpush")
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("prec,n,mode", [
+    (1, 152 * 128 - 1, "steady"), (1, 152 * 128, "steady"), (1, 152 * 128 + 1, "steady"), (1, 152 * 256 + 33, "steady"),
+    (1, 152 * 384 + 1, "steady"), (1, 152 * 128 + 1, "time"), (1, 152 * 256 + 1, "time"),
+    (0, 152 * 48 + 1, "steady"), (0, 152 * 128 + 1, "steady"), (0, 129, "time"),
+])
+def test_block_sizes_equal_one_thread_per_particle(prec, n, mode):
+    nodes = synth.wind_grid(WIND, dtype=np.float64 if prec == 0 else np.float32)
+    a, ta, sa = _run(prec, nodes, n, mode)
+    b, tb, sb = _run(prec, nodes, n, mode, grid_waves=0, block=32)
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
+    for k in ta:
+        assert np.array_equal(ta[k], tb[k]), k
+    for k in ("collisions", "rebirths", "flags_or", "particle_steps"):
+        assert sa[k] == sb[k], k
+
+
+def test_pushes_of_several_contexts_share_the_sms():
+    """Four contexts of 152 x 128 FP32 particles, one warp per scheduler each, on their own
+    streams: the four together against one alone. A step of a lone warp is its chain of some
+    2400 cycles for 850 instructions, so four on a scheduler take up to 3400, 1.4 times one
+    alone; four times where they run one after the other. The line is drawn at 2.5."""
+    nodes = synth.wind_grid(WIND, dtype=np.float32)
+    steps, ctxs = 20000, []
+    for k in range(4):
+        c = gcpush.Context(seed=k, stream=torch.cuda.Stream())
+        c.field_load(nodes, WIND.r_min_au, WIND.r_max_au)
+        c.inject([synth.EnsembleSpec(152 * 128, lam_au=0.5, r_out_au=synth.r_out_default(WIND))])
+        c.set_launch(steps_per_launch=steps)
+        c.advance(0.5, 100)
+        ctxs.append(c)
+
+    def timed(cs):
+        th = [threading.Thread(target=c.advance, args=(0.5, steps)) for c in cs]
+        t0 = time.perf_counter()
+        for t in th:
+            t.start()
+        for t in th:
+            t.join()
+        return time.perf_counter() - t0
+
+    one, four = [], []
+    for _ in range(4):
+        one.append(timed(ctxs[:1]))
+        four.append(timed(ctxs))
+    for c in ctxs:
+        c.close()
+    print("one %.1f ms, four %.1f ms" % (1e3 * min(one), 1e3 * min(four)))
+    assert min(four) < 2.5 * min(one)
