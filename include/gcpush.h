@@ -230,10 +230,13 @@ int gc_stats(gc_ctx *ctx, gc_stats_out *out);
  * checkpoint written with gc_particles_get; tally cadence and birth times follow them. */
 int gc_set_clock(gc_ctx *ctx, double t, int64_t step);
 
-/* Launch shape: threads per block (multiple of 32 up to 128; 0 = keep), steps per kernel
+/* Launch shape: threads per block (multiple of 32 up to 128; 0 = keep; GC_BLOCK_OWN = the
+ * library's own choice again, as in a new context), steps per kernel
  * launch (0 = keep), the period of the cell sort in steps (0 = never), and the grid in
  * resident waves of blocks (k >= 1: k x SMs x resident blocks per SM, each thread walking
- * several particles; 0: one thread per particle). */
+ * several particles; 0: one thread per particle). The library's own choice, with one wave, is
+ * one block per SM and, for few particles in FP64, four threads per particle. */
+enum { GC_BLOCK_OWN = -1 };
 int gc_set_launch(gc_ctx *ctx, int block, int steps_per_launch, int sort_every, int grid_waves);
 
 /* Replay gc_advance from CUDA graphs (enable != 0). The first call of a given pattern

@@ -182,7 +182,7 @@ struct gc_ctx {
     double field_ms = 0.0;
 
     // launch shape
-    int block = 0;           // 0: see push_block
+    int block = 0;           // 0: the library's own shape (push_block, quads)
     int grid_waves = 1;      // resident waves of blocks (0: one thread per particle)
     int blocks_per_sm[17] = {}; // occupancy per block size / 32, cached
     int steps_per_launch = 2000;
@@ -1070,11 +1070,11 @@ int gc_set_launch(gc_ctx *c, int block, int steps_per_launch, int sort_every, in
 {
     if (!c)
         return fail(GC_ERR_INVALID, "gc_set_launch: null context");
-    if (block != 0 && (block < 32 || block > 128 || block % 32 != 0))
+    if (block != 0 && block != GC_BLOCK_OWN && (block < 32 || block > 128 || block % 32 != 0))
         return fail(GC_ERR_INVALID, "gc_set_launch: block must be a multiple of 32 in [32, 128]");
     if (steps_per_launch < 0 || sort_every < 0 || grid_waves < 0)
         return fail(GC_ERR_INVALID, "gc_set_launch: negative argument");
-    if (block) c->block = block;
+    if (block) c->block = block == GC_BLOCK_OWN ? 0 : block;
     if (steps_per_launch) c->steps_per_launch = steps_per_launch;
     c->sort_every = sort_every;
     c->grid_waves = grid_waves;

@@ -28,6 +28,7 @@ GC_OK = 0
 GC_ERR = {-1: "GC_ERR_INVALID", -2: "GC_ERR_CUDA", -3: "GC_ERR_NOMEM", -4: "GC_ERR_STATE",
           -5: "GC_ERR_DEVICE_ANOMALY", -6: "GC_ERR_UNSUPPORTED"}
 PREC_FP64, PREC_FP32_MIXED = 0, 1
+BLOCK_OWN = -1
 DTYPE_F64, DTYPE_F32 = 0, 1
 
 
@@ -345,6 +346,7 @@ class Context:
 
     def set_launch(self, block: int = 0, steps_per_launch: int = 0, sort_every: int = 0,
                    grid_waves: int = 1):
+        """Launch shape; ``block``: threads per block, 0 keeps it, BLOCK_OWN is the library's choice."""
         _check(load().gc_set_launch(self._h, block, steps_per_launch, sort_every, grid_waves),
                "gc_set_launch")
 

@@ -1,6 +1,7 @@
 """The push's own launch shape for populations that do not fill the SMs: a block has as many
 threads as the population needs, so that several contexts' pushes run side by side, and no
 particle is lost or advanced twice at the edges between block sizes."""
+import statistics
 import threading
 import time
 
@@ -64,3 +65,39 @@ def test_pushes_of_several_contexts_share_the_sms():
         c.close()
     print("one %.1f ms, four %.1f ms" % (1e3 * min(one), 1e3 * min(four)))
     assert min(four) < 2.5 * min(one)
+
+
+def _push_ms(c, steps=200):
+    """Median push time of `steps` steps over a few calls."""
+    ms = []
+    for _ in range(5):
+        m = c.stats()["push_ms"]
+        c.advance(0.5, steps)
+        ms.append(c.stats()["push_ms"] - m)
+    return statistics.median(ms)
+
+
+def _fp64_4096():
+    c = gcpush.Context(precision=gcpush.PREC_FP64, seed=3)
+    c.field_load(synth.wind_grid(WIND, dtype=np.float64), WIND.r_min_au, WIND.r_max_au)
+    c.inject([synth.EnsembleSpec(4096, lam_au=0.5, r_out_au=synth.r_out_default(WIND))])
+    c.advance(0.5, 50)
+    return c
+
+
+def test_the_librarys_own_shape_can_be_asked_for_again():
+    """FP64 and 4096 particles: the library's own shape takes four threads per particle, which
+    measured 1.6 times as fast as blocks of 64 or 128; after such a block it has to be back."""
+    with _fp64_4096() as c:
+        own = _push_ms(c)
+        c.set_launch(block=64)
+        small = _push_ms(c)
+        c.set_launch()  # keeps the block
+        kept = _push_ms(c)
+        c.set_launch(block=gcpush.BLOCK_OWN)
+        again = _push_ms(c)
+        for bad in (-2, -32, 16, 48 + 1, 160, 512):
+            with pytest.raises(gcpush.GcError):
+                c.set_launch(block=bad)
+        print(own, small, kept, again)
+        assert min(small, kept) > 1.3 * own and again < 1.1 * own
