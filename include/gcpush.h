@@ -250,11 +250,13 @@ int gc_set_graph(gc_ctx *ctx, int enable);
 typedef struct {
     int32_t block, grid_waves, steps_per_launch, sort_every;
     double particle_steps_per_s; /* measured rate of the chosen shape */
-    int32_t trials, pad0;
+    int32_t trials;
+    int32_t own_shape;           /* 1: the library's own shape (GC_BLOCK_OWN) is the choice, and
+                                  * block the one of gc_set_launch's that is nearest to it */
 } gc_launch_choice;
 
-/* Time trial_steps steps of dt for each launch shape of a small search space (block size,
- * grid waves, cell-sort period) from a snapshot of the current state, keep the fastest
+/* Time trial_steps steps of dt for each launch shape of a small search space (the library's
+ * own shape and others by block size and grid waves; cell-sort period) from a snapshot of the current state, keep the fastest
  * with gc_set_launch, and restore the state, clock, counters and tallies as they were. */
 int gc_autotune(gc_ctx *ctx, double dt, int64_t trial_steps, gc_launch_choice *best);
 

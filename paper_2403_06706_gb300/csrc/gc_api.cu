@@ -1196,44 +1196,47 @@ int gc_autotune(gc_ctx *c, double dt, int64_t trial_steps, gc_launch_choice *bes
     gc_launch_choice b{};
     b.particle_steps_per_s = -1.0;
     int trials = 0;
-    const int blocks[] = {64, 128};
-    const int waves[] = {1, 2, 4, 0};
+    // The library's own shape first (block 0; it stands for one wave of blocks of 128, which it
+    // spreads the same way in larger blocks), then blocks of 64 and 128.
+    const int shapes[][2] = {{0, 1}, {64, 1}, {64, 2}, {64, 4}, {64, 0}, {128, 2}, {128, 4}, {128, 0}};
     const int sorts[] = {0, 250, 1000};
-    for (int blk : blocks) {
-        for (int wv : waves) {
-            for (int se : sorts) {
-                if (rc != GC_OK) break;
-                c->block = blk;
-                c->grid_waves = wv;
-                c->sort_every = se;
-                c->steps_per_launch = (int)std::min<int64_t>(trial_steps, 2000);
-                c->steps_since_sort = se; // a trial with sorting starts with one sort
-                rc = copy_state(c->st, bk, c->n, c->cap, c->stream);
-                if (rc != GC_OK) break;
-                const double push0 = c->push_ms, sort0 = c->sort_ms;
-                LaunchCounts lc;
-                rc = enqueue_advance(c, c->stream, dt, trial_steps, 0.0, nullptr, nullptr, &lc);
-                if (rc != GC_OK) break;
-                add_counts(c, lc);
-                bool an = false;
-                rc = collect_status(c, &an);
-                if (rc != GC_OK) break;
-                const double push_s = (c->push_ms - push0) * 1e-3;
-                const double sort_s = (c->sort_ms - sort0) * 1e-3;
-                // a sort serves sort_every steps: charge its share to this trial
-                const double per_step = push_s / trial_steps + (se > 0 ? sort_s / se : 0.0);
-                const double rate = (double)c->n / per_step;
-                ++trials;
-                if (rate > b.particle_steps_per_s) {
-                    b.block = blk;
-                    b.grid_waves = wv;
-                    b.sort_every = se;
-                    b.steps_per_launch = 2000;
-                    b.particle_steps_per_s = rate;
-                }
+    auto trial = [&](int blk, int wv, int se, double *rate) -> int {
+        c->block = blk;
+        c->grid_waves = wv;
+        c->sort_every = se;
+        c->steps_per_launch = (int)std::min<int64_t>(trial_steps, 2000);
+        c->steps_since_sort = se; // a trial with sorting starts with one sort
+        TRY(copy_state(c->st, bk, c->n, c->cap, c->stream));
+        const double push0 = c->push_ms, sort0 = c->sort_ms;
+        LaunchCounts lc;
+        TRY(enqueue_advance(c, c->stream, dt, trial_steps, 0.0, nullptr, nullptr, &lc));
+        add_counts(c, lc);
+        bool an = false;
+        TRY(collect_status(c, &an));
+        const double push_s = (c->push_ms - push0) * 1e-3, sort_s = (c->sort_ms - sort0) * 1e-3;
+        // a sort serves sort_every steps: charge its share to this trial
+        *rate = (double)c->n / (push_s / trial_steps + (se > 0 ? sort_s / se : 0.0));
+        return GC_OK;
+    };
+    double rate = 0.0;
+    // the kernels are loaded before the first timed trial
+    if (rc == GC_OK && (gcp::preload_kernels() != cudaSuccess || gcp::sort_preload() != cudaSuccess))
+        rc = fail(GC_ERR_CUDA, "gc_autotune: %s", cudaGetErrorString(cudaGetLastError()));
+    if (rc == GC_OK) rc = trial(0, 1, 0, &rate);
+    for (const auto &sh : shapes)
+        for (int se : sorts) {
+            if (rc == GC_OK) rc = trial(sh[0], sh[1], se, &rate);
+            if (rc != GC_OK) break;
+            ++trials;
+            if (rate > b.particle_steps_per_s) {
+                b.own_shape = sh[0] == 0;
+                b.block = sh[0] ? sh[0] : 128;
+                b.grid_waves = sh[1];
+                b.sort_every = se;
+                b.steps_per_launch = 2000;
+                b.particle_steps_per_s = rate;
             }
         }
-    }
     if (rc == GC_OK)
         rc = copy_state(c->st, bk, c->n, c->cap, c->stream);
     cudaStreamSynchronize(c->stream);
@@ -1255,7 +1258,7 @@ int gc_autotune(gc_ctx *c, double dt, int64_t trial_steps, gc_launch_choice *bes
         c->sort_every = se_sv;
         return rc;
     }
-    c->block = b.block;
+    c->block = b.own_shape ? 0 : b.block;
     c->grid_waves = b.grid_waves;
     c->steps_per_launch = b.steps_per_launch;
     c->sort_every = b.sort_every;

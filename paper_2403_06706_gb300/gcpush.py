@@ -149,7 +149,7 @@ FIELD_GRID, FIELD_SIREN, FIELD_GRID_SAMPLED = 0, 1, 2
 class LaunchChoice(C.Structure):
     _fields_ = [("block", C.c_int32), ("grid_waves", C.c_int32), ("steps_per_launch", C.c_int32),
                 ("sort_every", C.c_int32), ("particle_steps_per_s", C.c_double),
-                ("trials", C.c_int32), ("pad0", C.c_int32)]
+                ("trials", C.c_int32), ("own_shape", C.c_int32)]
 
 
 EXPORTS = ("gc_create", "gc_destroy", "gc_last_error", "gc_field_load", "gc_particles_inject",
@@ -356,7 +356,7 @@ class Context:
     def autotune(self, dt: float, trial_steps: int = 200) -> dict:
         b = LaunchChoice()
         _check(load().gc_autotune(self._h, dt, int(trial_steps), C.byref(b)), "gc_autotune")
-        return {k: getattr(b, k) for k, _ in LaunchChoice._fields_ if k != "pad0"}
+        return {k: getattr(b, k) for k, _ in LaunchChoice._fields_}
 
     def sort(self):
         _check(load().gc_sort(self._h), "gc_sort")

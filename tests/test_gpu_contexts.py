@@ -101,3 +101,38 @@ def test_the_librarys_own_shape_can_be_asked_for_again():
                 c.set_launch(block=bad)
         print(own, small, kept, again)
         assert min(small, kept) > 1.3 * own and again < 1.1 * own
+
+
+def test_autotune_keeps_four_threads_per_particle():
+    """FP64 and few particles: no block is as fast as the library's own shape (1.6 times)."""
+    with _fp64_4096() as c:
+        own = _push_ms(c)
+        best = c.autotune(0.5, trial_steps=100)
+        tuned = _push_ms(c)
+        print(best, own, tuned)
+        assert best["own_shape"] == 1 and best["block"] in (64, 128) and best["trials"] == 24
+        assert tuned < 1.1 * own
+
+
+def test_autotunes_choice_is_no_slower_than_the_default():
+    """64 uneven ensembles: the choice against a context's own launch shape, in turn, each over
+    1000 steps with the sorts they ask for. Two runs of one shape differ by up to 3 %."""
+    wl = synth.c3_batched()
+    nodes = synth.wind_grid(wl.wind, dtype=np.float32)
+    with gcpush.Context(precision=gcpush.PREC_FP32_MIXED, seed=wl.seed) as c:
+        c.field_load(nodes, wl.wind.r_min_au, wl.wind.r_max_au)
+        c.inject(list(wl.ensembles))
+        c.advance(wl.dt, 500)
+        best = c.autotune(wl.dt, trial_steps=200)
+        block = gcpush.BLOCK_OWN if best["own_shape"] else best["block"]
+        ms = {"own": [], "tuned": []}
+        for _ in range(5):
+            for name, shape in (("own", dict(block=gcpush.BLOCK_OWN)),
+                                ("tuned", dict(block=block, sort_every=best["sort_every"], grid_waves=best["grid_waves"]))):
+                c.set_launch(steps_per_launch=2000, **shape)
+                a = c.stats()
+                c.advance(wl.dt, 1000)
+                b = c.stats()
+                ms[name].append(b["push_ms"] + b["sort_ms"] - a["push_ms"] - a["sort_ms"])
+    print(best, ms)
+    assert statistics.median(ms["tuned"]) < 1.03 * statistics.median(ms["own"])
