@@ -48,13 +48,6 @@ __device__ __forceinline__ void p2_split(unsigned long long v, float &lo, float 
     asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
 
-__device__ __forceinline__ unsigned long long p2_add(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // Sine and cosine of two values at once, for |z| <= kSincosMax: Cody and Waite's reduction
 // r = z - q pi/2 (q = z 2/pi rounded to an integer by adding 1.5 2^23, pi/2 in three parts)
 // and minimal-error polynomials on |r| <= pi/4 (fitted by sincos_coeffs.py). At most 1.55 ulp
