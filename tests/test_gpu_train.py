@@ -122,3 +122,28 @@ def test_gradient_into_a_slice_of_a_flat_buffer(off):
         assert abs(c.siren_loss_grad(x, t, view) - loss) < 1e-12 * loss
     assert float((view - g).norm()) < 1e-5 * float(g.norm()) > 0.0
     assert bool((flat[:off] == 7.0).all()) and bool((flat[off + gcpush.SIREN_NPARAMS:] == 7.0).all())
+
+
+def test_gradient_of_a_large_batch_is_the_mean_of_its_parts():
+    """2^22 samples against the mean over eight parts, summed in FP64. Sums in tensor memory are
+    rounded towards zero: terms of one sign (targets of a common mean) lose up to 1e-7 of the
+    gradient per 64 samples added there, 2.6e-4 between the whole and its parts where each of
+    25 splits of the batch is one such sum. Rounded to nearest instead, the 2622 additions of a
+    split and the 25 of the splits leave sqrt(2647 / 3) 2^-25, 1e-6. Held to 4e-6."""
+    n, parts = 1 << 22, 8
+    g = torch.Generator(device="cuda").manual_seed(4)
+    x = torch.rand((n, 3), generator=g, device="cuda") * 1.2 - 0.6
+    t = torch.randn((n, 8), generator=g, device="cuda") * 0.3 + 0.5
+    whole = torch.empty(gcpush.SIREN_NPARAMS, device="cuda")
+    with gcpush.Context() as c:
+        c.siren_set(synth.siren_init(seed=9), omega0=30.0)
+        c.siren_loss_grad(x, t, whole)
+        mean = torch.zeros(gcpush.SIREN_NPARAMS, dtype=torch.float64, device="cuda")
+        part = torch.empty_like(whole)
+        for xs, ts in zip(x.chunk(parts), t.chunk(parts)):
+            c.siren_loss_grad(xs, ts, part)
+            mean += part.double() / parts
+    hidden = slice(1024, 198400)
+    err = float((whole.double() - mean)[hidden].norm() / mean[hidden].norm())
+    print(err)
+    assert err < 4e-6
