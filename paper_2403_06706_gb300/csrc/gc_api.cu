@@ -437,7 +437,7 @@ int enqueue_advance(gc_ctx *c, cudaStream_t s, double dt, int64_t n_steps, doubl
             TRY(do_sort(c, s, owned, lc));
             P.st = c->st;
         }
-        int64_t chunk = std::min<int64_t>(n_steps - done, c->steps_per_launch);
+        int64_t chunk = std::min<int64_t>(n_steps - done, std::min(c->steps_per_launch, 1 << 30));
         if (c->sort_every > 0)
             chunk = std::min<int64_t>(chunk, std::max<int64_t>(1, c->sort_every - c->steps_since_sort));
         P.step0 = c->step + done;

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__((kPushThreads<T, TD>), 1) push_kernel(const __
         PConst c;
         PState<T> s;
         load_particle(P, i, c, s);
-        int next_tally = INT32_MAX - 1; // the step that ends on the next tally sample
+        int next_tally = kNoTally; // the step that ends on the next tally sample
         if (P.tally_on) {
             const int64_t K = P.tally.cadence;
             next_tally = (int)((K - 1 - (step0 % K)) % K);
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__((kPushThreads<T, TD>), 1) push_kernel(const __
                 ++k;
             }
             if (k == next_tally + 1) {
-                next_tally += P.tally.cadence;
+                next_tally = after_tally(next_tally, P.tally.cadence);
                 const double t_new = step_time(t0, (long long)(P.kbase + k), P.dt);
                 tally_sample<T>(P.tally, P, ph, c.e, AccOf<T>::val(s.Rx), AccOf<T>::val(s.Ry), AccOf<T>::val(s.Rz),
                                 AccOf<T>::val(s.U), s.mub, s.Bm0, t_new - s.t_birth, s.ncoll,
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(32, 1) push_quad_kernel(const __grid_constant_
     uint32_t event = P.st.event[i], ncoll = P.st.ncoll[i], flags = P.st.flags[i];
     unsigned n_coll = 0, n_reb = 0;
 
-    int next_tally = INT32_MAX - 1;
+    int next_tally = kNoTally;
     if (P.tally_on) {
         const int64_t K = P.tally.cadence;
         next_tally = (int)((K - 1 - (step0 % K)) % K);
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(32, 1) push_quad_kernel(const __grid_constant_
             ++k;
         }
         if (k == next_tally + 1) {
-            next_tally += P.tally.cadence;
+            next_tally = after_tally(next_tally, P.tally.cadence);
             const double x = q_get(A, 0), y = q_get(A, 1), z = q_get(A, 2), u = q_get(A, 3);
             const double t_new = step_time(t0, (long long)(P.kbase + k), P.dt);
             tally_sample<double>(P.tally, P, ph, e, x, y, z, u, mub, Bm0, t_new - t_birth, ncoll,

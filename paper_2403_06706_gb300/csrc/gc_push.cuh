@@ -110,6 +110,15 @@ __device__ __forceinline__ void agg_inc64(unsigned long long *base, int idx)
         atomicAdd(base + idx, (unsigned long long)__popc(grp));
 }
 
+// Step of a launch that ends on the next tally sample (the loops run up to the step after it),
+// and the one a cadence later: none in this launch where that is beyond an int (a cadence near
+// 2^31 stands for "never").
+constexpr int kNoTally = INT32_MAX - 1;
+__device__ __forceinline__ int after_tally(int next, int cadence)
+{
+    return cadence < kNoTally - next ? next + cadence : kNoTally;
+}
+
 // Snapshot sample of one particle (Sect. 3). FP64: the bins are computed with the same
 // operations as the definition (double); FP32: the same formulas in float, with
 // gamma - 1 formed without cancellation.
