@@ -54,9 +54,11 @@ constexpr uint32_t kW5Bytes = 4u * 16u * 128u; // W5 padded to 16 rows: 4 boxes 
 // fast ones differ from them in the last place; where that moves a BF16 rounding, everything
 // behind it in the sample is rounded anew, and the gradient moves by 8e-4 / sqrt(samples):
 // 3.5e-5 for 512, 4e-6 for 32768 (either is 2e-3 from the gradient in FP64, BF16's rounding).
-// So that small batches, which are bound by the chain's latency, take the same roundings as
-// plain sinf and cosf: within 1.3e-6. At 512 samples 71 us for loss and gradient (215 with
-// a pass over memory per layer), at 16384 132 (395), at 32768 with the fast ones 169 (541).
+// So that small batches take the same roundings as plain sinf and cosf, and keep the results
+// that they have always had: within 1.3e-6. That is what the line is for; it is neither the
+// faster side (loss and gradient of 128, 4096, 8192, 16384 samples 70.5, 82, 94, 130 us here, 62,
+// 70, 82, 107 with the fast ones; 215 at 512 and 395 at 16384 with a pass over memory per layer)
+// nor the more accurate one (rms error of sine and cosine on |z| <= 30 1.9e-8 here, 1.7e-8 there).
 constexpr int64_t kLibrarySines = 16384;
 constexpr int kStagesPerTile = 24;             // 6 products x 4
 constexpr int kComputeThreads = 512;
@@ -613,12 +615,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 // one accumulator, and while the next chunk's MMAs fill the other (2 x 256 columns), eight warps
 // add it to FP32 sums in registers, rounded to nearest. 2^22 samples against
 // the mean of eight parts: 2.3e-7 (2.6e-4 with one such sum per split of the batch). The drains
-// hide behind the operands' copies, which bound the kernel: loss and gradient of 65536 samples
-// 270 us with chunks of 1, 2 or 4 stages, 268 without them.
+// hide behind the operands' copies, which bound the kernel (one batch of a fit, 8192 and 65536
+// samples: 89.3 and 264.5 us, as with one sum per split), once the sums leave by whole rows:
+// added to the gradient straight from the registers, in sectors of 32 rows, 91.4 and 266.8.
 constexpr int kDwStages = 4;
 constexpr int kDwChunk = 2;
 constexpr int kDwSumWarps = 8, kDwThreads = 32 * (kDwSumWarps + 1); // the last warp issues
 constexpr uint32_t kDwStageBytes = (128u + 256u) * 128u;
+constexpr int kDwPitch = 260; // floats per row of the sums on their way out: no bank conflicts
+static_assert(128 * kDwPitch * 4 <= kDwStages * kDwStageBytes, "the sums fit in the stages");
 constexpr size_t kSmemDw = kDwStages * kDwStageBytes + 1024 + 256;
 
 __global__ void __launch_bounds__(kDwThreads, 1)
@@ -740,12 +745,24 @@ __global__ void __launch_bounds__(kDwThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(&drained[b]);
         }
+        // the sums leave by rows of 1024 bytes, through the stages that are free now (every load
+        // landed and was consumed before the last chunk's signal)
+        float *const rows = (float *)smem;
         if (ok) {
-            float *dst = G + siren_oW(L + 2) + (int64_t)(m0 + (warp & 3) * 32 + lane) * 256 + (warp >> 2) * 128;
+            float *dst = rows + ((warp & 3) * 32 + lane) * kDwPitch + (warp >> 2) * 128;
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-                atomicAdd(reinterpret_cast<float4 *>(dst) + j,
-                          make_float4(sum[4 * j], sum[4 * j + 1], sum[4 * j + 2], sum[4 * j + 3]));
+                reinterpret_cast<float4 *>(dst)[j] = make_float4(sum[4 * j], sum[4 * j + 1], sum[4 * j + 2], sum[4 * j + 3]);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kDwSumWarps) : "memory");
+        if (ok && !*abort) {
+            float *dst = G + siren_oW(L + 2) + (int64_t)m0 * 256;
+#pragma unroll 4
+            for (int r = warp; r < 128; r += kDwSumWarps)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    atomicAdd(reinterpret_cast<float4 *>(dst + r * 256 + h * 128) + lane,
+                              reinterpret_cast<const float4 *>(rows + r * kDwPitch + h * 128)[lane]);
         }
     }
     tc_fence_before();
