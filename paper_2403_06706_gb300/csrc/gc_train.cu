@@ -18,11 +18,12 @@
 // one launch, both operands K-major in that layout; the batch is split so that the CTAs of
 // all layers fill the SMs once, and the splits add up by FP32 atomics.
 //
-// What bounds kernel 1: the tile is one dependent chain of 13 steps, about 48 000 cycles, of
-// which the CUDA cores' own work (sine and cosine of 4 x 256 pre-activations per sample at
-// library accuracy, dW5) is about 30 000 and the tensor cores' 10 000 (a 128 x 64 x 16 MMA
-// takes 48 cycles: shared memory). 203 us of 270 us for loss and gradient of 65536 samples;
-// kernel 2 takes 41 us, reading 300 MB, two thirds of them from memory. Before, each layer made passes over
+// What bounds kernel 1: the tile is one dependent chain of 13 steps, about 56 000 cycles (203 us
+// for the seven rounds of tiles of 65536 samples at 1.95 GHz). In it the CUDA cores issue 87 000
+// warp instructions (sine and cosine of 4 x 256 pre-activations per sample, dW5), 21 700 slots of
+// each scheduler, and the tensor cores take 10 000 cycles (a 128 x 64 x 16 MMA takes 48: shared
+// memory). 203 us of 271 us for loss and gradient; kernel 2 takes 40 us, reading 300 MB, two
+// thirds of them from memory. Before, each layer made passes over
 // [sample][256] buffers (FP32 pre-activations, their gradients: 2 GB of traffic): 905 us.
 // Warp roles of kernel 1 (608 threads): warps 0-15 compute (warp w: features 32 (w % 4) +
 // lane of a half, samples 16 (w / 4) ..), warp 16 issues MMAs, warp 17 TMA loads of the
